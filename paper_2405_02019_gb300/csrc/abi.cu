@@ -255,10 +255,14 @@ void enqueue_graph_steps(snn_net *net, int64_t m, cudaStream_t st)
 }
 
 // Pipelined engine: m step kernels from step t0 (the device's t_base), every circuit
-// group in turn, then t_base += m.  Consecutive kernels of a group may overlap their
-// launch with the previous one (programmatic edges, inside a captured graph); a group's
-// first kernel follows the previous group's resync in plain stream order.
-int enqueue_pipelined_steps(snn_net *net, int64_t m, cudaStream_t st, int64_t t0, bool programmatic)
+// group in turn, then t_base += m.  Consecutive kernels of a group overlap their launch
+// with the previous one (programmatic edges), inside a captured graph and launched one by
+// one alike; a group's first kernel follows the previous group's resync (or the previous
+// run's k_advance, whose t_base it reads before waiting) in plain stream order.
+// One-by-one launches without the edges took 6.2 us per step at pd_full and at pd_tiny,
+// against 3.5 and 3.3 in a graph: a kernel boundary in plain order drains the GPU, and the
+// next kernel's launch and its network, table and Philox work then sit on the chain.
+int enqueue_pipelined_steps(snn_net *net, int64_t m, cudaStream_t st, int64_t t0)
 {
     const size_t G = net->group_args.size();
     for (size_t g = 0; g < std::max<size_t>(G, 1); ++g) {
@@ -266,7 +270,7 @@ int enqueue_pipelined_steps(snn_net *net, int64_t m, cudaStream_t st, int64_t t0
         const int grid = G ? net->group_grid[g] : net->step_grid;
         for (int64_t k = 0; k < m; ++k) {
             const int ph = static_cast<int>((t0 + k) % snn::kPhasePeriod);
-            const int e = snn::launch_step(a, static_cast<int>(k), ph, grid, st, programmatic && k > 0);
+            const int e = snn::launch_step(a, static_cast<int>(k), ph, grid, st, k > 0);
             if (e != 0) return fail(SNN_ECUDA, std::string("step launch: ") + cudaGetErrorString(static_cast<cudaError_t>(e)));
         }
         if (g + 1 < G) snn::launch_resync(net->args.ctl, st);
@@ -279,7 +283,7 @@ int enqueue_pipelined_steps(snn_net *net, int64_t m, cudaStream_t st, int64_t t0
 int launch_steps_direct(snn_net *net, int64_t m, cudaStream_t st, int64_t t0)
 {
     if (net->engine == SNN_ENGINE_PIPELINED) {
-        const int rc = enqueue_pipelined_steps(net, m, st, t0, false);
+        const int rc = enqueue_pipelined_steps(net, m, st, t0);
         if (rc) return rc;
     } else {
         enqueue_graph_steps(net, m, st);
@@ -328,7 +332,7 @@ int capture_graph(snn_net *net)
     SNN_CUDA_TRY(cudaStreamBeginCapture(net->capture_stream, cudaStreamCaptureModeThreadLocal));
     if (net->engine == SNN_ENGINE_PIPELINED) {
         // replays start on a multiple of the phase period (see snn_step_n)
-        const int rc = enqueue_pipelined_steps(net, net->steps_per_graph, net->capture_stream, 0, true);
+        const int rc = enqueue_pipelined_steps(net, net->steps_per_graph, net->capture_stream, 0);
         if (rc != SNN_OK) {
             cudaGraph_t g = nullptr;
             cudaStreamEndCapture(net->capture_stream, &g);

@@ -630,8 +630,8 @@ __device__ __forceinline__ void pipe_deliver(const StepArgs &a, const int64_t &t
         pipe_deliver_fmt<SNN_RECORD_PLAIN9, kGroup>(a, t, ph, dw, ndw, n, rbase, first);
 }
 
-// t_base is read before waiting on the previous kernel: within a graph replay it only
-// changes in the replay's last node, and direct launches are not programmatic.
+// t_base is read before waiting on the previous kernel: it only changes in the k_advance
+// that ends a run of steps, and a run's first kernel is not a programmatic launch.
 template <bool kGroup>
 __global__ void __launch_bounds__(kStepMaxThreads, 2) k_step(const StepArgs a, const int k, const int ph)
 {
