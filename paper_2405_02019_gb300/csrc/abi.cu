@@ -72,8 +72,6 @@ struct snn_net {
     cudaStream_t capture_stream = nullptr;
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t graph_exec = nullptr;
-    cudaEvent_t ev_done = nullptr;
-    bool ev_recorded = false;
     int64_t t = 0;
     uint32_t device_error = 0;
     // drained raster, ordered by (step, neuron)
@@ -82,11 +80,14 @@ struct snn_net {
     int64_t events_read = 0;
     int32_t *pin_nrn = nullptr, *pin_t = nullptr;
     int64_t pin_cap = 0;
-    // overlapped reads: every snn_step_n ends by copying the device raster cursor into
-    // snap_cursor[call mod kSnaps] (pinned) and recording snap_ev there; raster_read is
-    // the device raster index up to which spikes are already in the host history
+    // every snn_step_n ends by copying the device raster cursor and the error bits (four
+    // words of Ctl from the cursor on) into snap_ctl[call mod kSnaps] (pinned) and recording
+    // snap_ev there; raster_read is the device raster index up to which spikes are already
+    // in the host history
     static constexpr int kSnaps = 4;
-    uint32_t *snap_cursor = nullptr;
+    uint32_t *snap_ctl = nullptr;
+    bool snap_fresh = false;       // the latest snapshot is where the device stands when it is done
+    bool drained = false;          // nothing was enqueued since the last drain
     cudaEvent_t snap_ev[kSnaps] = {};
     int64_t snap_t[kSnaps] = {};   // steps enqueued at each snapshot
     int64_t n_snaps = 0;           // snapshots recorded
@@ -366,25 +367,86 @@ int recapture(snn_net *net)
 
 int wait_done(snn_net *net)
 {
-    if (net->ev_recorded) SNN_CUDA_TRY(cudaEventSynchronize(net->ev_done));
+    if (net->n_snaps > 0) SNN_CUDA_TRY(cudaEventSynchronize(net->snap_ev[(net->n_snaps - 1) % snn_net::kSnaps]));
     return SNN_OK;
 }
 
-// Raster entries [lo, hi) of the device raster into the host history, ordered by
-// (step, neuron), through the handle's copy stream (the steps that wrote them are done).
-int append_raster(snn_net *net, int64_t lo, int64_t hi)
+// Pinned staging for at least `want` entries of each of the raster's two arrays.
+int reserve_pinned(snn_net *net, int64_t want)
+{
+    if (want <= net->pin_cap) return SNN_OK;
+    if (net->pin_nrn) cudaFreeHost(net->pin_nrn);
+    if (net->pin_t) cudaFreeHost(net->pin_t);
+    net->pin_nrn = net->pin_t = nullptr;
+    net->pin_cap = 0;
+    want = std::max<int64_t>(want, 1 << 16);
+    SNN_CUDA_TRY(cudaMallocHost(&net->pin_nrn, sizeof(int32_t) * want));
+    SNN_CUDA_TRY(cudaMallocHost(&net->pin_t, sizeof(int32_t) * want));
+    net->pin_cap = want;
+    return SNN_OK;
+}
+
+// The stretch [lo, hi) of the device raster, whose steps lie in [t_lo, t_hi), ordered on
+// the device (raster.cu) into the pinned staging: neurons in pin_nrn, and in pin_t where
+// each step's neurons start (t_hi - t_lo + 2 offsets).  `ok` is false if a spike's step was
+// outside the range.
+int order_on_device(snn_net *net, int64_t lo, int64_t hi, int64_t t_lo, int64_t t_hi, bool &ok)
+{
+    snn::RasterSort a{};
+    a.t = reinterpret_cast<const int32_t *>(net->arena + net->L.rast_t) + lo;
+    a.nrn = reinterpret_cast<const int32_t *>(net->arena + net->L.rast_nrn) + lo;
+    a.count = hi - lo;
+    a.t0 = t_lo;
+    a.n_steps = t_hi - t_lo;
+    a.cur = reinterpret_cast<uint32_t *>(net->arena + net->L.sort_cur);
+    a.off = reinterpret_cast<uint32_t *>(net->arena + net->L.sort_off);
+    a.out = reinterpret_cast<int32_t *>(net->arena + net->L.sort_out);
+    int dev = 0;
+    SNN_CUDA_TRY(cudaGetDevice(&dev));
+    if (dev != net->device) SNN_CUDA_TRY(cudaSetDevice(net->device));
+    const int e = snn::launch_raster_sort(a, net->num_sms, net->copy_stream);
+    if (dev != net->device) SNN_CUDA_TRY(cudaSetDevice(dev));
+    if (e != 0) return fail(SNN_ECUDA, std::string("raster order: ") + cudaGetErrorString(static_cast<cudaError_t>(e)));
+    SNN_CUDA_TRY(cudaMemcpyAsync(net->pin_t, a.off, 4 * (a.n_steps + 2), cudaMemcpyDeviceToHost, net->copy_stream));
+    SNN_CUDA_TRY(cudaMemcpyAsync(net->pin_nrn, a.out, 4 * a.count, cudaMemcpyDeviceToHost, net->copy_stream));
+    SNN_CUDA_TRY(cudaStreamSynchronize(net->copy_stream));
+    const uint32_t *off = reinterpret_cast<const uint32_t *>(net->pin_t);
+    ok = off[a.n_steps] == off[a.n_steps + 1];
+    for (int64_t s = 0; ok && s < a.n_steps; ++s)
+        if (off[s + 1] - off[s] > static_cast<uint32_t>(snn::kRasterMaxBucket))
+            std::sort(net->pin_nrn + off[s], net->pin_nrn + off[s + 1]);
+    return SNN_OK;
+}
+
+// Raster entries [lo, hi) of the device raster, spikes of steps [t_lo, t_hi), into the host
+// history, ordered by (step, neuron), through the handle's copy stream (the steps that
+// wrote them are done).  With `idle` (no step is running) more than kRasterSortMin spikes
+// are ordered on the device; while steps run they are ordered on the host, because the
+// resident engine's CTAs fill the SMs until their call ends.
+int append_raster(snn_net *net, int64_t lo, int64_t hi, int64_t t_lo, int64_t t_hi, bool idle)
 {
     const int64_t cnt = hi - lo;
     if (cnt <= 0) return SNN_OK;
-    if (cnt > net->pin_cap) {
-        if (net->pin_nrn) cudaFreeHost(net->pin_nrn);
-        if (net->pin_t) cudaFreeHost(net->pin_t);
-        net->pin_nrn = net->pin_t = nullptr;
-        net->pin_cap = 0;
-        const int64_t want = std::max<int64_t>(cnt, 1 << 16);
-        SNN_CUDA_TRY(cudaMallocHost(&net->pin_nrn, sizeof(int32_t) * want));
-        SNN_CUDA_TRY(cudaMallocHost(&net->pin_t, sizeof(int32_t) * want));
-        net->pin_cap = want;
+    const bool on_device = idle && cnt >= snn::kRasterSortMin && cnt <= snn::kRasterSortMax && t_hi > t_lo &&
+                           t_hi - t_lo <= snn::kRasterSortMaxSteps;
+    int rc = reserve_pinned(net, std::max(cnt, on_device ? t_hi - t_lo + 2 : 0));
+    if (rc) return rc;
+    // room first (growing by at least half), so that nothing below can fail half-way
+    const size_t base = net->hist_t.size();
+    for (auto *v : {&net->hist_t, &net->hist_i})
+        if (v->capacity() < base + cnt) v->reserve(std::max<size_t>(base + cnt, v->capacity() + v->capacity() / 2));
+    if (on_device) {
+        bool ok = false;
+        rc = order_on_device(net, lo, hi, t_lo, t_hi, ok);
+        if (rc) return rc;
+        if (ok) {
+            const uint32_t *off = reinterpret_cast<const uint32_t *>(net->pin_t);
+            net->hist_i.insert(net->hist_i.end(), net->pin_nrn, net->pin_nrn + cnt);
+            for (int64_t s = 0; s < t_hi - t_lo; ++s)
+                net->hist_t.insert(net->hist_t.end(), off[s + 1] - off[s], static_cast<int32_t>(t_lo + s));
+            for (int64_t j = 0; j < cnt; ++j) net->events_read += net->out_degree[net->pin_nrn[j]];
+            return SNN_OK;
+        }
     }
     const int32_t *dn = reinterpret_cast<const int32_t *>(net->arena + net->L.rast_nrn) + lo;
     const int32_t *dt = reinterpret_cast<const int32_t *>(net->arena + net->L.rast_t) + lo;
@@ -422,43 +484,59 @@ int append_raster(snn_net *net, int64_t lo, int64_t hi)
     }
     // the range covers whole steps after every step already in the history (a snapshot
     // ends an snn_step_n call), so appending keeps the history ordered
-    const size_t base = net->hist_t.size();
-    net->hist_t.resize(base + cnt);
-    net->hist_i.resize(base + cnt);
     for (int64_t j = 0; j < cnt; ++j) {
-        net->hist_t[base + j] = static_cast<int32_t>(key[j] >> 32);
         const int32_t i = static_cast<int32_t>(key[j] & 0xFFFFFFFFll);
-        net->hist_i[base + j] = i;
+        net->hist_t.push_back(static_cast<int32_t>(key[j] >> 32));
+        net->hist_i.push_back(i);
         net->events_read += net->out_degree[i];
     }
     return SNN_OK;
 }
 
 // Waits for every enqueued step, moves the rest of the device raster to the host
-// history and resets the device cursor.
-int drain(snn_net *net)
+// history and resets the device cursor.  Where the cursor and the error bits stand is
+// known from the last call's snapshot; a drain with nothing enqueued since the last one
+// touches the device no more.
+int drain_steps(snn_net *net)
 {
     int rc = wait_done(net);
     if (rc) return rc;
-    snn::Ctl ctl;
-    SNN_CUDA_TRY(cudaMemcpy(&ctl, net->arena + net->L.ctl, sizeof(ctl), cudaMemcpyDeviceToHost));
-    net->device_error |= ctl.err;
-    const int64_t cnt = std::min<int64_t>(ctl.cursor, net->L.rast_cap);
-    rc = append_raster(net, std::min(net->raster_read, cnt), cnt);
-    if (rc) return rc;
-    if (ctl.cursor != 0) {
-        uint32_t zero[3] = {0, 0, 0};  // cursor, step_begin[0], step_begin[1]
-        SNN_CUDA_TRY(cudaMemcpy(net->arena + net->L.ctl + offsetof(snn::Ctl, cursor), zero, sizeof(zero),
-                                cudaMemcpyHostToDevice));
+    if (!net->drained) {
+        uint32_t end[4];  // Ctl: cursor, step_begin[2], err
+        if (net->snap_fresh) {
+            std::memcpy(end, net->snap_ctl + 4 * ((net->n_snaps - 1) % snn_net::kSnaps), sizeof(end));
+        } else {
+            SNN_CUDA_TRY(cudaMemcpy(end, net->arena + net->L.ctl + offsetof(snn::Ctl, cursor), sizeof(end),
+                                    cudaMemcpyDeviceToHost));
+        }
+        net->device_error |= end[3];
+        const int64_t cnt = std::min<int64_t>(end[0], net->L.rast_cap);
+        rc = append_raster(net, std::min(net->raster_read, cnt), cnt, net->collected_t, net->t, true);
+        if (rc) return rc;
+        net->raster_read = cnt;  // a failed reset below leaves the entries read once
+        net->collected_t = net->t;
+        if (end[0] != 0) {  // cursor, step_begin[0], step_begin[1]
+            SNN_CUDA_TRY(cudaMemsetAsync(net->arena + net->L.ctl + offsetof(snn::Ctl, cursor), 0, 12, net->copy_stream));
+            SNN_CUDA_TRY(cudaStreamSynchronize(net->copy_stream));
+        }
+        net->raster_read = 0;
+        net->snaps_valid_from = net->n_snaps;  // their cursors refer to the raster before the reset
+        net->drained = true;
     }
-    net->raster_read = 0;
-    net->snaps_valid_from = net->n_snaps;  // their cursors refer to the raster before the reset
-    net->collected_t = net->t;
     if (net->device_error & snn::kErrTimeout)
         return fail(SNN_ETIMEOUT, "a bounded device wait (persistent barrier or resident mailbox) timed out");
     if (net->device_error & snn::kErrRaster)
         return fail(SNN_EOVERFLOW, "device raster filled before it was read; raise raster_capacity");
     return SNN_OK;
+}
+
+int drain(snn_net *net)
+{
+    try {
+        return drain_steps(net);
+    } catch (const std::bad_alloc &) {
+        return fail(SNN_ENOMEM, "host allocation failed while reading spikes");
+    }
 }
 
 // Moves the spikes of the calls before the latest snn_step_n into the host history
@@ -471,10 +549,15 @@ int collect(snn_net *net)
     if (j < 0 || j < net->snaps_valid_from) return SNN_OK;
     const int slot = static_cast<int>(j % snn_net::kSnaps);
     SNN_CUDA_TRY(cudaEventSynchronize(net->snap_ev[slot]));
-    const int64_t cur = net->snap_cursor[slot];
+    const int64_t cur = net->snap_ctl[4 * slot];
     if (cur > net->L.rast_cap / 4) return drain(net);
-    const int rc = append_raster(net, net->raster_read, std::max(net->raster_read, cur));
-    if (rc) return rc;
+    try {
+        const int rc = append_raster(net, net->raster_read, std::max(net->raster_read, cur), net->collected_t,
+                                     std::max(net->collected_t, net->snap_t[slot]), false);
+        if (rc) return rc;
+    } catch (const std::bad_alloc &) {
+        return fail(SNN_ENOMEM, "host allocation failed while reading spikes");
+    }
     net->raster_read = std::max(net->raster_read, cur);
     net->collected_t = std::max(net->collected_t, net->snap_t[slot]);
     return SNN_OK;
@@ -864,12 +947,10 @@ int snn_build_network(const snn_spec *spec, void *dev_arena, uint64_t arena_byte
             }
         }
         rc = (net->engine == SNN_ENGINE_GRAPH || net->engine == SNN_ENGINE_PIPELINED) ? capture_graph(net) : SNN_OK;
-        if (rc == SNN_OK && cudaEventCreateWithFlags(&net->ev_done, cudaEventDisableTiming) != cudaSuccess)
-            rc = fail(SNN_ECUDA, "event create");
         for (int k = 0; k < snn_net::kSnaps && rc == SNN_OK; ++k)
             if (cudaEventCreateWithFlags(&net->snap_ev[k], cudaEventDisableTiming) != cudaSuccess)
                 rc = fail(SNN_ECUDA, "event create");
-        if (rc == SNN_OK && cudaMallocHost(&net->snap_cursor, sizeof(uint32_t) * snn_net::kSnaps) != cudaSuccess)
+        if (rc == SNN_OK && cudaMallocHost(&net->snap_ctl, 4 * sizeof(uint32_t) * snn_net::kSnaps) != cudaSuccess)
             rc = fail(SNN_ECUDA, "pinned snapshot slots");
         if (rc == SNN_OK && cudaStreamCreateWithFlags(&net->copy_stream, cudaStreamNonBlocking) != cudaSuccess)
             rc = fail(SNN_ECUDA, "copy stream");
@@ -893,6 +974,8 @@ int snn_step_n(snn_net *net, int64_t n_steps, void *cuda_stream)
     if (net->device_error) return fail(SNN_ESTATE, "a previous device error is pending");
     if (n_steps == 0) return SNN_OK;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    net->drained = false;
+    net->snap_fresh = false;
     if (net->engine == SNN_ENGINE_PERSISTENT || net->engine == SNN_ENGINE_RESIDENT) {
         const int rc = net->engine == SNN_ENGINE_RESIDENT ? launch_steps_resident(net, n_steps, st)
                                                           : launch_steps_persistent(net, n_steps, st);
@@ -916,16 +999,15 @@ int snn_step_n(snn_net *net, int64_t n_steps, void *cuda_stream)
             if (rc) return rc;
         }
     }
-    SNN_CUDA_TRY(cudaEventRecord(net->ev_done, st));
-    net->ev_recorded = true;
     net->t += n_steps;
-    // where the raster ends after these steps, for snn_collect_spikes
+    // where the raster and the error bits stand after these steps
     const int slot = static_cast<int>(net->n_snaps % snn_net::kSnaps);
-    SNN_CUDA_TRY(cudaMemcpyAsync(net->snap_cursor + slot, net->arena + net->L.ctl + offsetof(snn::Ctl, cursor),
-                                 sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
+    SNN_CUDA_TRY(cudaMemcpyAsync(net->snap_ctl + 4 * slot, net->arena + net->L.ctl + offsetof(snn::Ctl, cursor),
+                                 4 * sizeof(uint32_t), cudaMemcpyDeviceToHost, st));
     SNN_CUDA_TRY(cudaEventRecord(net->snap_ev[slot], st));
     net->snap_t[slot] = net->t;
     net->n_snaps += 1;
+    net->snap_fresh = true;
     return SNN_OK;
 }
 
@@ -936,6 +1018,8 @@ int snn_profile_steps(snn_net *net, int64_t n_steps, void *cuda_stream, double *
     if (n_steps < 0) return fail(SNN_EINVAL, "n_steps < 0");
     if (net->device_error) return fail(SNN_ESTATE, "a previous device error is pending");
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    net->drained = false;
+    net->snap_fresh = false;
     if (net->engine == SNN_ENGINE_RESIDENT) {
         // one cooperative launch runs both phases of every step: its time goes to ms_update
         cudaEvent_t e0, e1;
@@ -1234,6 +1318,8 @@ int snn_load_state(snn_net *net, const void *host_buf, uint64_t bytes)
         return fail(SNN_EINVAL, "state was saved from a network of another shape or engine");
     int rc = wait_done(net);
     if (rc) return rc;
+    net->drained = false;
+    net->snap_fresh = false;
     const uint8_t *in = static_cast<const uint8_t *>(host_buf);
     uint64_t off = sizeof(h);
     for (const auto &sg : seg) {
@@ -1372,14 +1458,13 @@ int snn_deliver_spikes(snn_net *net, const int32_t *spikers, int64_t n_spikers, 
 void snn_destroy(snn_net *net)
 {
     if (!net) return;
-    if (net->ev_recorded) cudaEventSynchronize(net->ev_done);
+    if (net->n_snaps > 0) cudaEventSynchronize(net->snap_ev[(net->n_snaps - 1) % snn_net::kSnaps]);
     if (net->graph_exec) cudaGraphExecDestroy(net->graph_exec);
     if (net->graph) cudaGraphDestroy(net->graph);
     if (net->capture_stream) cudaStreamDestroy(net->capture_stream);
-    if (net->ev_done) cudaEventDestroy(net->ev_done);
     for (int k = 0; k < snn_net::kSnaps; ++k)
         if (net->snap_ev[k]) cudaEventDestroy(net->snap_ev[k]);
-    if (net->snap_cursor) cudaFreeHost(net->snap_cursor);
+    if (net->snap_ctl) cudaFreeHost(net->snap_ctl);
     if (net->copy_stream) cudaStreamDestroy(net->copy_stream);
     if (net->pin_nrn) cudaFreeHost(net->pin_nrn);
     if (net->pin_t) cudaFreeHost(net->pin_t);

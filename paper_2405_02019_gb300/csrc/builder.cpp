@@ -342,6 +342,10 @@ Layout make_layout(const snn_spec &spec)
     L.pop_id = o; o = up(o + L.npad);
     L.group_circuit = o; o = up(o + 4 * (L.npad / 128 + 1));
     L.circuits = o; o = up(o + sizeof(CircuitInfo) * std::max(1, spec.n_circuits));
+    // scratch of the raster's ordering: per-step counters and offsets, the ordered neurons
+    L.sort_cur = o; o = up(o + 4 * (kRasterSortMaxSteps + 1));
+    L.sort_off = o; o = up(o + 4 * (kRasterSortMaxSteps + 2));
+    L.sort_out = o; o = up(o + 4 * std::min(L.rast_cap, kRasterSortMax));
     L.total = o;
     return L;
 }

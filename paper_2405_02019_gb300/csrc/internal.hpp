@@ -213,6 +213,22 @@ struct StepArgs {
     int32_t res_stride;           // resident engine: shared ring row stride (widest block, multiple of 32)
 };
 
+// Ordering of a stretch of the raster on the device (raster.cu).
+constexpr int kRasterMaxBucket = 8192;                     // spikes of one step ordered in shared memory
+// Fewer spikes are ordered on the host, at about 15 ns each where the device's launches
+// cost about 20 us (a read of 267 spikes takes 37 us, one of 3,870 takes 72 us).
+constexpr int64_t kRasterSortMin = 2048;
+constexpr int64_t kRasterSortMax = int64_t{1} << 22;       // spikes of one stretch (the scratch's size) ...
+constexpr int64_t kRasterSortMaxSteps = int64_t{1} << 17;  // ... and the steps it covers
+struct RasterSort {
+    const int32_t *t, *nrn;  // the stretch: steps and neurons
+    int64_t count;
+    int64_t t0, n_steps;     // every spike's step is in [t0, t0 + n_steps)
+    uint32_t *cur;           // scratch [n_steps + 1]
+    uint32_t *off;           // out [n_steps + 2]: where each step's neurons start; the last is count
+    int32_t *out;            // out [count]: neurons by (step, neuron)
+};
+
 // Host constants of one model (§2.2).
 struct Constants {
     double w_f, p11, p22, beta, gamma, p21;
@@ -253,7 +269,7 @@ struct HostNetwork {
 // Arena layout for a spec.
 struct Layout {
     uint64_t ctl, tables, U, I, R, ring, row_ptr, syn_tgt, syn_w, syn_d, rast_nrn, rast_t, U2, R2, queue, qcount, pop_id,
-        group_circuit, circuits, blocks, seg, mbox, inbox, res_rec, total;
+        group_circuit, circuits, blocks, seg, mbox, inbox, res_rec, sort_cur, sort_off, sort_out, total;
     int64_t npad, syn_padded_max, rast_cap;
 };
 
@@ -292,6 +308,9 @@ void launch_prime(const StepArgs &a, int grid, void *stream);         // pipelin
 int prepare_step_kernel(const StepArgs &a);                           // dynamic shared memory opt-in
 int step_grid(int num_sms, int64_t quad_warps);  // default CTAs of the step kernel
 int step_threads(const StepArgs &a);
+
+// raster.cu: the stretch ordered by (step, neuron)
+int launch_raster_sort(const RasterSort &a, int num_sms, void *stream);
 
 // resident.cu
 // Block width of the resident engine for n neurons on num_sms SMs (a multiple of
