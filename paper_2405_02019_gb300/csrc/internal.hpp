@@ -97,10 +97,8 @@ constexpr int kBlockAvgWidth = 512;          // sets the number of in-degree quo
 constexpr int kBlockAlign = 32;              // block boundaries are multiples of 32
 constexpr int kBlockQuad = 4;                // (row, block) segments are whole quads of records
 constexpr int kBlockedThreads = 1024;
-constexpr int kBlockedBatch = 2048;          // senders staged per pass
-constexpr int kBlockedWindow = 8192;         // quads of a pass whose record-array index is tabled at once
-constexpr int kBlockedBinDelays = 32;        // delays summed in shared memory (longer: ring reductions)
-constexpr int kBlockedRounds = 4;            // quads in flight per lane (32 per round and warp)
+constexpr int kBlockedBinRows = 48;           // delays below this are summed in shared memory (longer: ring reductions)
+constexpr int kBlockedBinDelays = 32;         // the same for block-major records
 constexpr int64_t kBlockedAggregateMin = 64; // fewer senders: reduce straight into the ring
 inline int max_target_blocks(int64_t n)
 {
@@ -215,9 +213,7 @@ struct StepArgs {
 
 // Ordering of a stretch of the raster on the device (raster.cu).
 constexpr int kRasterMaxBucket = 8192;                     // spikes of one step ordered in shared memory
-// Fewer spikes are ordered on the host, at about 15 ns each where the device's launches
-// cost about 20 us (a read of 267 spikes takes 37 us, one of 3,870 takes 72 us).
-constexpr int64_t kRasterSortMin = 2048;
+constexpr int64_t kRasterSortMin = 2048;                   // fewer spikes: ordered on the host
 constexpr int64_t kRasterSortMax = int64_t{1} << 22;       // spikes of one stretch (the scratch's size) ...
 constexpr int64_t kRasterSortMaxSteps = int64_t{1} << 17;  // ... and the steps it covers
 struct RasterSort {
@@ -293,10 +289,6 @@ void launch_advance(Ctl *ctl, int64_t m, void *stream);
 // circuit groups: the next group starts the same steps where the raster now ends
 void launch_resync(Ctl *ctl, void *stream);
 void launch_deliver_list(const StepArgs &a, const int32_t *list, int64_t n, int64_t t, int grid, void *stream);
-// blocked records: one CTA per target block; list == nullptr delivers step t_base + k's
-// spikes from the raster (graph engine), else list[0 .. n) as spikes of step t
-int prepare_blocked_kernel();
-void launch_deliver_blocked(const StepArgs &a, const int32_t *list, int64_t n, int64_t t, int k, void *stream);
 int deliver_list_blocks_per_sm();
 int update_grid(int64_t n);  // CTAs of k_update for n neurons
 int persistent_blocks_per_sm(const StepArgs &a);
@@ -308,6 +300,11 @@ void launch_prime(const StepArgs &a, int grid, void *stream);         // pipelin
 int prepare_step_kernel(const StepArgs &a);                           // dynamic shared memory opt-in
 int step_grid(int num_sms, int64_t quad_warps);  // default CTAs of the step kernel
 int step_threads(const StepArgs &a);
+
+// blocked.cu: one CTA per target block; list == nullptr delivers step t_base + k's
+// spikes from the raster (graph engine), else list[0 .. n) as spikes of step t
+int prepare_blocked_kernel();
+void launch_deliver_blocked(const StepArgs &a, const int32_t *list, int64_t n, int64_t t, int k, void *stream);
 
 // raster.cu: the stretch ordered by (step, neuron)
 int launch_raster_sort(const RasterSort &a, int num_sms, void *stream);
