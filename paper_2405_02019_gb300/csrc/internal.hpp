@@ -98,7 +98,6 @@ constexpr int kBlockAlign = 32;              // block boundaries are multiples o
 constexpr int kBlockQuad = 4;                // (row, block) segments are whole quads of records
 constexpr int kBlockedThreads = 1024;
 constexpr int kBlockedBinRows = 48;           // delays below this are summed in shared memory (longer: ring reductions)
-constexpr int kBlockedBinDelays = 32;         // the same for block-major records
 constexpr int64_t kBlockedAggregateMin = 64; // fewer senders: reduce straight into the ring
 inline int max_target_blocks(int64_t n)
 {
