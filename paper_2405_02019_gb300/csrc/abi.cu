@@ -55,6 +55,7 @@ struct snn_net {
     int32_t max_row = 0, chunks_per_row = 1;
     std::vector<int64_t> pop_off;
     std::vector<int32_t> out_degree;
+    snn::SlicePlan slices{};  // phase 2 alone on rows, for long lists (parts = 0: none)
     int format = SNN_RECORD_PLAIN9;
     std::vector<uint8_t> pop_id;
     std::vector<snn::CircuitInfo> circuits;
@@ -780,6 +781,13 @@ int snn_build_network(const snn_spec *spec, void *dev_arena, uint64_t arena_byte
             cuda_ok(cudaMemcpyAsync(A + L.syn_w, hn.wbytes.data(), hn.wbytes.size(), cudaMemcpyHostToDevice, st),
                     "weights");
         }
+        if (!hn.row_delay.empty()) {
+            cuda_ok(cudaMemcpyAsync(A + L.row_delay, hn.row_delay.data(), 2 * hn.row_delay.size(), cudaMemcpyHostToDevice,
+                                    st), "row delays");
+            net->slices = snn::make_slice_plan(hn.delay_events, net->n, net->npad);
+            if (net->slices.parts > 0)
+                cuda_ok(static_cast<cudaError_t>(snn::prepare_slices_kernel(hn.format)), "slices kernel");
+        }
         cuda_ok(cudaStreamSynchronize(st), "upload sync");
         if (rc != SNN_OK) {
             delete net;
@@ -809,6 +817,7 @@ int snn_build_network(const snn_spec *spec, void *dev_arena, uint64_t arena_byte
         a.pop_id = A + L.pop_id;
         a.group_circuit = reinterpret_cast<const int32_t *>(A + L.group_circuit);
         a.circuits = reinterpret_cast<const snn::CircuitInfo *>(A + L.circuits);
+        a.row_delay = reinterpret_cast<const uint16_t *>(A + L.row_delay);
         a.blk_rec = reinterpret_cast<const uint16_t *>(A + L.syn_tgt);
         a.blk_seg = reinterpret_cast<const uint16_t *>(A + L.syn_d);
         a.blk_off = reinterpret_cast<const int32_t *>(A + L.blocks);
@@ -1447,6 +1456,12 @@ int snn_deliver_spikes(snn_net *net, const int32_t *spikers, int64_t n_spikers, 
     if (snn::is_blocked(net->format)) {
         snn::launch_deliver_blocked(net->args, spikers, n_spikers, t, 0, cuda_stream);
         SNN_CUDA_TRY(cudaGetLastError());
+        return SNN_OK;
+    }
+    // long lists go slice by slice, unless the caller sets the launch's CTAs
+    if (blocks == 0 && snn::slices_pay(net->slices, n_spikers, n_spikers * (net->n_syn / net->n))) {
+        const int e = snn::launch_deliver_slices(net->args, net->slices, spikers, n_spikers, t, net->num_sms, cuda_stream);
+        if (e != 0) return fail(SNN_ECUDA, std::string("deliver: ") + cudaGetErrorString(static_cast<cudaError_t>(e)));
         return SNN_OK;
     }
     const int grid = blocks > 0 ? blocks : net->num_sms * snn::deliver_list_blocks_per_sm();

@@ -13,6 +13,7 @@
 //
 // Built with -ffp-contract=off: every FP64 product and sum is rounded on its own.
 #include <algorithm>
+#include <array>
 #include <atomic>
 #include <cmath>
 #include <cstring>
@@ -346,6 +347,8 @@ Layout make_layout(const snn_spec &spec)
     L.sort_cur = o; o = up(o + 4 * (kRasterSortMaxSteps + 1));
     L.sort_off = o; o = up(o + 4 * (kRasterSortMaxSteps + 2));
     L.sort_out = o; o = up(o + 4 * std::min(L.rast_cap, kRasterSortMax));
+    // where each delay starts in every row (the layouts that keep rows in delay order)
+    L.row_delay = o; o = up(o + (is_blocked(fmt) || resident ? 0 : 2 * uint64_t{kDMax} * n));
     L.total = o;
     return L;
 }
@@ -779,6 +782,7 @@ bool build_host_network(const snn_spec &spec, const Constants &c, HostNetwork &n
         all.d.reserve(s_all);
     }
     int64_t base = 0;
+    bool delay_table = true;
     for (int ci = 0; ci < spec.n_circuits; ++ci) {
         snn_spec one = circuit_spec(spec, ci);
         one.record_format = SNN_RECORD_PLAIN9;
@@ -794,6 +798,14 @@ bool build_host_network(const snn_spec &spec, const Constants &c, HostNetwork &n
             all.u0.push_back(0.0f);
             all.pop_id.push_back(0);
             ++all.n;
+        }
+        delay_table = delay_table && !h.row_delay.empty();
+        if (delay_table) {
+            all.row_delay.resize(static_cast<size_t>(all.n) * kDMax, 0);  // the gap's empty rows
+            all.row_delay.insert(all.row_delay.end(), h.row_delay.begin(), h.row_delay.end());
+            for (int k = 0; k < kDMax; ++k) all.delay_events[k] += h.delay_events[k];
+        } else {
+            std::vector<uint16_t>().swap(all.row_delay);
         }
         for (int64_t i = 0; i < h.n; ++i) {
             all.row_ptr.push_back(syn_base + h.row_ptr[i + 1]);
@@ -927,7 +939,12 @@ bool build_one(const snn_spec &spec, const Constants &c, HostNetwork &net, std::
     net.tgt.assign(net.n_syn_padded, 0);
     net.w.assign(net.n_syn_padded, 0);
     net.d.assign(net.n_syn_padded, 1);
-    parallel_for(nthreads, n, [&](int, int64_t lo, int64_t hi) {
+    // where each delay starts in its row, and the synapses of each delay, for the layouts
+    // that keep the delay order (16-bit offsets: no longer rows)
+    const bool delay_table = !is_blocked(spec.record_format) && spec.engine != SNN_ENGINE_RESIDENT && maxrow <= 65535;
+    if (delay_table) net.row_delay.resize(static_cast<size_t>(n) * kDMax);
+    std::vector<std::array<int64_t, kDMax>> delay_events(std::max(1, nthreads), std::array<int64_t, kDMax>{});
+    parallel_for(nthreads, n, [&](int th, int64_t lo, int64_t hi) {
         int64_t cnt[kDMax];
         for (int64_t i = lo; i < hi; ++i) {
             std::fill(cnt, cnt + kDMax, 0);
@@ -935,6 +952,10 @@ bool build_one(const snn_spec &spec, const Constants &c, HostNetwork &net, std::
             int64_t pos = net.row_ptr[i];
             for (int k = 0; k < kDMax; ++k) {
                 const int64_t c0 = cnt[k];
+                if (delay_table) {
+                    if (k > 0) net.row_delay[static_cast<size_t>(i) * kDMax + k] = static_cast<uint16_t>(pos - net.row_ptr[i]);
+                    delay_events[th][k] += c0;
+                }
                 cnt[k] = pos;
                 pos += c0;
             }
@@ -944,6 +965,7 @@ bool build_one(const snn_spec &spec, const Constants &c, HostNetwork &net, std::
                 net.w[dst] = s_w[s];
                 net.d[dst] = s_d[s];
             }
+            if (delay_table) net.row_delay[static_cast<size_t>(i) * kDMax] = static_cast<uint16_t>(pos - net.row_ptr[i]);
             // padding entries: zero weight onto the sender itself, delay 1
             for (int64_t s = pos; s < net.row_ptr[i + 1]; ++s) {
                 net.tgt[s] = static_cast<int32_t>(i);
@@ -952,6 +974,8 @@ bool build_one(const snn_spec &spec, const Constants &c, HostNetwork &net, std::
             }
         }
     });
+    for (const auto &ev : delay_events)
+        for (int k = 0; k < kDMax; ++k) net.delay_events[k] += ev[k];
     net.pop_id.assign(n, 0);
     for (int b = 0; b < m.n_pops; ++b)
         for (int64_t i = net.pop_off[b]; i < net.pop_off[b + 1]; ++i) net.pop_id[i] = static_cast<uint8_t>(b);

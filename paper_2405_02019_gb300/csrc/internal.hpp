@@ -206,8 +206,21 @@ struct StepArgs {
     const void *res_rec;          // resident engine: block-major int2 records {weight, local target | delay << 16}
     int32_t res_lens_stride;
     int32_t res_coarse_stride;
+    const uint16_t *row_delay;    // rows in delay order: [n][64], where each delay starts in its row (entry 0: the row's end)
     int32_t res_rows;             // resident engine: ring rows kept in shared memory (power of two, 8..64)
     int32_t res_stride;           // resident engine: shared ring row stride (widest block, multiple of 32)
+};
+
+// Phase 2 alone for long lists on rows, one slice of delays per CTA (slices.cu).
+constexpr int32_t kSliceCells = 40960;           // sums in a CTA's shared memory
+constexpr int kSliceMaxParts = 2;                // target ranges that a network may be cut into
+struct SlicePlan {
+    int32_t parts;   // target ranges (0: no plan) ...
+    int32_t width;   // ... of this many neurons
+    int32_t delays;  // delays per group
+    int32_t tail;    // the delays from here on form the last group, reduced directly
+    int32_t groups;
+    uint32_t cum[kDMax + 1];  // the groups' bounds on the line of work
 };
 
 // Ordering of a stretch of the raster on the device (raster.cu).
@@ -254,6 +267,8 @@ struct HostNetwork {
     std::vector<int32_t> w;
     std::vector<uint8_t> d;
     std::vector<float> u0;
+    std::vector<uint16_t> row_delay;  // rows in delay order: [n][64] where each delay starts, entry 0 the row's end (empty if a row is too long)
+    int64_t delay_events[kDMax] = {}; // synapses of each delay
     std::vector<int32_t> blk;      // blocked records: block boundaries
     std::vector<uint16_t> rec16;   // blocked records: local target | delay << 10
     std::vector<uint16_t> seg;     // blocked records: [n][blocks + 1] block starts per row
@@ -264,7 +279,7 @@ struct HostNetwork {
 // Arena layout for a spec.
 struct Layout {
     uint64_t ctl, tables, U, I, R, ring, row_ptr, syn_tgt, syn_w, syn_d, rast_nrn, rast_t, U2, R2, queue, qcount, pop_id,
-        group_circuit, circuits, blocks, seg, mbox, inbox, res_rec, sort_cur, sort_off, sort_out, total;
+        group_circuit, circuits, blocks, seg, mbox, inbox, res_rec, sort_cur, sort_off, sort_out, row_delay, total;
     int64_t npad, syn_padded_max, rast_cap;
 };
 
@@ -304,6 +319,13 @@ int step_threads(const StepArgs &a);
 // spikes from the raster (graph engine), else list[0 .. n) as spikes of step t
 int prepare_blocked_kernel();
 void launch_deliver_blocked(const StepArgs &a, const int32_t *list, int64_t n, int64_t t, int k, void *stream);
+
+// slices.cu: list[0 .. n) as spikes of step t, on rows with a delay table
+bool slices_pay(const SlicePlan &plan, int64_t n_senders, int64_t events);
+SlicePlan make_slice_plan(const int64_t (&events)[kDMax], int64_t n, int64_t npad);
+int prepare_slices_kernel(int format);
+int launch_deliver_slices(const StepArgs &a, const SlicePlan &plan, const int32_t *list, int64_t n, int64_t t, int num_sms,
+                          void *stream);
 
 // raster.cu: the stretch ordered by (step, neuron)
 int launch_raster_sort(const RasterSort &a, int num_sms, void *stream);
