@@ -808,8 +808,9 @@ int snn_build_network(const snn_spec *spec, void *dev_arena, uint64_t arena_byte
         a.rast_nrn = reinterpret_cast<int32_t *>(A + L.rast_nrn);
         a.rast_t = reinterpret_cast<int32_t *>(A + L.rast_t);
         a.n = net->n;
+        a.n_all = net->n;
         a.npad = net->npad;
-        a.seed = spec->seed;
+        a.seed = net->circuits[0].seed;  // of the only circuit
         a.rast_cap = static_cast<uint32_t>(L.rast_cap);
         a.chunks_per_row = net->chunks_per_row;
         a.format = net->format;

@@ -165,7 +165,8 @@ struct StepArgs {
     const uint8_t *syn_d;
     int32_t *rast_nrn;
     int32_t *rast_t;
-    int64_t n;        // neurons
+    int64_t n;        // neurons (the launch's end neuron where a circuit group has its own)
+    int64_t n_all;    // neurons of the network
     int64_t npad;     // ring row stride
     uint64_t seed;
     uint32_t rast_cap;

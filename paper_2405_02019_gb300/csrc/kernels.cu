@@ -385,28 +385,11 @@ __device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes)
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
 }
 
-// Poisson count T = #{k : v >= thr[k]} (thresholds nondecreasing): the first eight
-// thresholds of the quad's population come in registers, the rest from memory.
-__device__ __forceinline__ uint32_t poisson_count(uint64_t v, const uint64_t (&r)[8], const uint64_t *thr_row)
-{
-    uint32_t T = 0;
-#pragma unroll
-    for (int k = 0; k < 8; ++k) T += (v >= r[k]) ? 1u : 0u;
-    if (T == 8u)
-        while (T < static_cast<uint32_t>(kPK) && v >= __ldg(thr_row + T)) ++T;
-    return T;
-}
-
 // Waits until the previous kernel of the stream has completed and its writes are
 // visible (a no-op unless this launch was made programmatic).
 __device__ __forceinline__ void wait_previous_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void allow_next_grid() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
-// Neuron part for quad q = 32 g + lane: B(t) (unless do_b is false: the first kernel,
-// t = -1) then A(t+1).  Warp-collective: every lane of group g must call it (lanes
-// without a quad pass valid = false).  Everything that does not depend on the
-// previous step (row bounds, Poisson thresholds, the Philox block) is done before
-// `wait_first` (if set) waits for the previous kernel.
 // A launch of one circuit group (kGroup) takes its queue counts, queue size and first
 // group of 128 neurons from the arguments; a launch over the whole index space uses the
 // control block's counts, npad entries per queue and group 0.  The two are separate
@@ -427,87 +410,108 @@ __device__ __forceinline__ int64_t first_quad_warp(const StepArgs &a)
     return kGroup ? (a.quad_base >> 5) : 0;
 }
 
-template <bool kGroup>
-__device__ __forceinline__ void pipe_quad(const StepArgs &a, const int64_t &t, int ph, int64_t g, bool valid,
-                                          bool do_b, bool wait_first)
+// The thalamic counts of four neurons, one byte each, from Philox counter (t, ctr): the
+// first eight thresholds of the first neuron's population are read once and compared with
+// all four words; a count of eight and more goes on from there, and a quad that spans two
+// populations looks each neuron's up.  Not inlined: the step kernel draws in two places.
+__device__ __noinline__ uint32_t draw_quad(uint64_t t, uint64_t ctr, uint64_t seed, uint32_t pops,
+                                           const uint64_t *thresholds)
 {
-    const int lane = threadIdx.x & 31;
-    const int64_t q = g * 32 + lane;
-    const int64_t i0 = q * 4;
-    const int phn = ph + 1;  // phase of the step whose spikes are decided here
-    int32_t spk[4] = {0, 0, 0, 0};
-    int64_t rp[5] = {0, 0, 0, 0, 0};
-    // independent of the previous step: network, tables, circuit, random numbers
-    uint64_t tr[8] = {0, 0, 0, 0, 0, 0, 0, 0};
-    Block4 rnd = {{0, 0, 0, 0}};
-    int b0 = 0;
-    uint32_t pops = 0;
-    int64_t end_valid = 0;  // neurons of the quad's circuit end here
-    const uint64_t *thr0 = a.tables->thresholds[0];
-    if (valid) {
-        const longlong2 rpa = __ldg(reinterpret_cast<const longlong2 *>(a.row_ptr + i0));
-        const longlong2 rpb = __ldg(reinterpret_cast<const longlong2 *>(a.row_ptr + i0 + 2));
-        const int64_t rpc = __ldg(a.row_ptr + i0 + 4);
-        rp[0] = rpa.x; rp[1] = rpa.y; rp[2] = rpb.x; rp[3] = rpb.y; rp[4] = rpc;
-        const CircuitInfo ci = a.circuits[__ldg(a.group_circuit + g)];
-        end_valid = ci.base + ci.n;
-        pops = __ldg(reinterpret_cast<const unsigned int *>(a.pop_id + i0));
-        b0 = pops & 0xFF;
-        thr0 = &a.tables->thresholds[b0][0];
-        if (do_b) {
+    const Block4 rnd = philox4x64_10(t, ctr, 0, 0, seed, kStreamThalamic);
+    const uint64_t *thr = thresholds + (pops & 0xFFu) * kPK;
+    uint32_t T[4] = {0, 0, 0, 0};
 #pragma unroll
-            for (int k = 0; k < 8; k += 2) {
-                const ulonglong2 v2 = __ldg(reinterpret_cast<const ulonglong2 *>(thr0 + k));
-                tr[k] = v2.x;
-                tr[k + 1] = v2.y;
-            }
-            rnd = philox4x64_10(static_cast<uint64_t>(t), static_cast<uint64_t>((i0 - ci.base) >> 2), 0, 0, ci.seed,
-                                kStreamThalamic);
-        }
-    }
-    if (wait_first) wait_previous_grid();
-    if (valid) {
-        const float *Uin = (ph & 1) ? a.U2 : a.U;
-        const uint8_t *Rin = (ph & 1) ? a.R2 : a.R;
-        float *Uout = (phn & 1) ? a.U2 : a.U;
-        uint8_t *Rout = (phn & 1) ? a.R2 : a.R;
-        // the state of the quad, in one round trip
-        const float4 u4 = *reinterpret_cast<const float4 *>(Uin + i0);
-        const float4 c4 = *reinterpret_cast<const float4 *>(a.I + i0);
-        const uint32_t r4 = *reinterpret_cast<const uint32_t *>(Rin + i0);
-        int32_t *wrow = a.ring + (ph & kDMask) * a.npad + i0;
-        int4 w4 = make_int4(0, 0, 0, 0);
-        if (do_b) w4 = __ldcg(reinterpret_cast<const int4 *>(wrow));
-        float uu[4] = {u4.x, u4.y, u4.z, u4.w};
-        float cc[4] = {c4.x, c4.y, c4.z, c4.w};
-        uint32_t rr[4] = {r4 & 0xFFu, (r4 >> 8) & 0xFFu, (r4 >> 16) & 0xFFu, r4 >> 24};
-        if (do_b) {
-            *reinterpret_cast<int4 *>(wrow) = make_int4(0, 0, 0, 0);
-            const int32_t ww[4] = {w4.x, w4.y, w4.z, w4.w};
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int64_t i = i0 + j;
-                if (i < end_valid) {
-                    const int b = (pops >> (8 * j)) & 0xFF;
-                    const uint64_t v = rnd.w[j] >> 1;
-                    uint32_t T;
-                    if (b == b0) {
-                        T = poisson_count(v, tr, thr0);
-                    } else {  // a population boundary inside the quad: read that row from memory
-                        const uint64_t *thr = &a.tables->thresholds[b][0];
-                        T = 0;
-                        while (T < static_cast<uint32_t>(kPK) && v >= __ldg(thr + T)) ++T;
-                    }
-                    const int32_t in =
-                        static_cast<int32_t>(static_cast<uint32_t>(ww[j]) + T * static_cast<uint32_t>(a.w_ext_fx));
-                    cc[j] = __fadd_rn(__fmul_rn(a.p11, cc[j]), __fmul_rn(__int2float_rn(in), 0x1p-12f));
-                }
-            }
-            *reinterpret_cast<float4 *>(a.I + i0) = make_float4(cc[0], cc[1], cc[2], cc[3]);
-        }
+    for (int k = 0; k < 8; k += 2) {
+        const ulonglong2 v2 = __ldg(reinterpret_cast<const ulonglong2 *>(thr + k));
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            if (i0 + j >= end_valid) continue;
+            const uint64_t v = rnd.w[j] >> 1;
+            T[j] += (v >= v2.x ? 1u : 0u) + (v >= v2.y ? 1u : 0u);
+        }
+    }
+    const bool mixed = pops != (pops & 0xFFu) * 0x01010101u;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if (!mixed && T[j] < 8u) continue;
+        const uint64_t v = rnd.w[j] >> 1;
+        const uint64_t *own = thresholds + ((pops >> (8 * j)) & 0xFFu) * kPK;
+        uint32_t c = mixed ? 0u : 8u;
+        while (c < static_cast<uint32_t>(kPK) && v >= __ldg(own + c)) ++c;
+        T[j] = c;
+    }
+    return T[0] | (T[1] << 8) | (T[2] << 16) | (T[3] << 24);
+}
+
+// The draws of step t for quad q = 32 g + lane (g: group of 128 neurons), one byte per neuron:
+// the thalamic count, and kDrawValid for a neuron of a circuit (the others are inert).
+// Independent of the dynamics, so a step kernel draws before it waits for the kernel before it.
+constexpr uint32_t kDrawValid = 0x80u;
+__device__ __forceinline__ uint32_t pipe_draws(const StepArgs &a, int64_t t, int64_t g, bool draw)
+{
+    const int64_t i0 = (g * 32 + (threadIdx.x & 31)) * 4;
+    if (g >= a.quad_warps || i0 >= a.n) return 0u;
+    CircuitInfo ci{0, a.n_all, a.seed, 0};
+    if (a.n_circuits > 1) ci = a.circuits[__ldg(a.group_circuit + g)];
+    uint32_t packed = 0;
+    if (draw)
+        packed = draw_quad(static_cast<uint64_t>(t), static_cast<uint64_t>((i0 - ci.base) >> 2), ci.seed,
+                           __ldg(reinterpret_cast<const unsigned int *>(a.pop_id + i0)), a.tables->thresholds[0]);
+    const int64_t left = ci.base + ci.n - i0;  // neurons of the circuit from the quad on
+    return left >= 4 ? packed | kDrawValid * 0x01010101u
+           : left > 0 ? packed | (kDrawValid * 0x01010101u >> (8 * (4 - left)))
+                      : packed;
+}
+
+// The dynamic state of a quad, loaded in one round trip.
+struct QuadState {
+    float4 u, c;
+    uint32_t r;
+    int4 w;
+};
+
+template <bool kB>
+__device__ __forceinline__ void pipe_load(const StepArgs &a, int ph, int64_t g, bool valid, QuadState &s)
+{
+    const int64_t i0 = (g * 32 + (threadIdx.x & 31)) * 4;
+    s.u = make_float4(0.f, 0.f, 0.f, 0.f);
+    s.c = s.u;
+    s.r = 0;
+    s.w = make_int4(0, 0, 0, 0);
+    if (!valid) return;
+    s.u = *reinterpret_cast<const float4 *>(((ph & 1) ? a.U2 : a.U) + i0);
+    s.c = *reinterpret_cast<const float4 *>(a.I + i0);
+    s.r = *reinterpret_cast<const uint32_t *>(((ph & 1) ? a.R2 : a.R) + i0);
+    if (kB) s.w = __ldcg(reinterpret_cast<const int4 *>(a.ring + (ph & kDMask) * a.npad + i0));
+}
+
+// Neuron part for quad q = 32 g + lane: B(t) (without kB, the first kernel: t = -1, not) then
+// A(t+1), from the quad's draws and state.  Warp-collective: every lane of group g must call
+// it (lanes without a quad pass valid = false).
+template <bool kGroup, bool kB>
+__device__ __forceinline__ void pipe_quad(const StepArgs &a, const int64_t &t, int ph, int64_t g, bool valid,
+                                          uint32_t draws, const QuadState &s)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t i0 = (g * 32 + lane) * 4;
+    const int phn = ph + 1;  // phase of the step whose spikes are decided here
+    int32_t spk[4] = {0, 0, 0, 0};
+    if (valid) {
+        float *Uout = (phn & 1) ? a.U2 : a.U;
+        uint8_t *Rout = (phn & 1) ? a.R2 : a.R;
+        float uu[4] = {s.u.x, s.u.y, s.u.z, s.u.w};
+        float cc[4] = {s.c.x, s.c.y, s.c.z, s.c.w};
+        const int32_t ww[4] = {s.w.x, s.w.y, s.w.z, s.w.w};
+        uint32_t rr[4] = {s.r & 0xFFu, (s.r >> 8) & 0xFFu, (s.r >> 16) & 0xFFu, s.r >> 24};
+        if (kB) *reinterpret_cast<int4 *>(a.ring + (ph & kDMask) * a.npad + i0) = make_int4(0, 0, 0, 0);
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint32_t draw = (draws >> (8 * j)) & 0xFFu;
+            if (!(draw & kDrawValid)) continue;
+            if (kB) {
+                const int32_t in = static_cast<int32_t>(static_cast<uint32_t>(ww[j]) +
+                                                        (draw & 0x7Fu) * static_cast<uint32_t>(a.w_ext_fx));
+                cc[j] = __fadd_rn(__fmul_rn(a.p11, cc[j]), __fmul_rn(__int2float_rn(in), 0x1p-12f));
+            }
             if (rr[j] == 0u) {
                 float x = __fadd_rn(__fmul_rn(a.p22, uu[j]), __fmul_rn(a.p21, cc[j]));
                 if (x >= a.theta) {
@@ -521,21 +525,29 @@ __device__ __forceinline__ void pipe_quad(const StepArgs &a, const int64_t &t, i
                 rr[j] -= 1u;
             }
         }
+        if (kB) *reinterpret_cast<float4 *>(a.I + i0) = make_float4(cc[0], cc[1], cc[2], cc[3]);
         *reinterpret_cast<float4 *>(Uout + i0) = make_float4(uu[0], uu[1], uu[2], uu[3]);
         *reinterpret_cast<uint32_t *>(Rout + i0) = rr[0] | (rr[1] << 8) | (rr[2] << 16) | (rr[3] << 24);
     }
-    // the group's spikes of step t+1: count and entries, plain stores in its own region
+    // the group's spikes of step t+1 into the queue: room from one atomic per warp, the
+    // spikers' row bounds in the same round trip
     const int cnt = spk[0] + spk[1] + spk[2] + spk[3];
+    if (!__any_sync(0xFFFFFFFFu, cnt != 0)) return;
+    int64_t rp[5] = {0, 0, 0, 0, 0};
+    if (cnt != 0) {
+        const longlong2 rpa = __ldg(reinterpret_cast<const longlong2 *>(a.row_ptr + i0));
+        const longlong2 rpb = __ldg(reinterpret_cast<const longlong2 *>(a.row_ptr + i0 + 2));
+        rp[0] = rpa.x; rp[1] = rpa.y; rp[2] = rpb.x; rp[3] = rpb.y;
+        rp[4] = __ldg(a.row_ptr + i0 + 4);
+    }
     int incl = cnt;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
         const int v = __shfl_up_sync(0xFFFFFFFFu, incl, o);
         if (lane >= o) incl += v;
     }
-    const int total = __shfl_sync(0xFFFFFFFFu, incl, 31);
-    if (total == 0) return;
     uint32_t base = 0;
-    if (lane == 31) base = atomicAdd(&queue_counts<kGroup>(a)[phn & 3], static_cast<uint32_t>(total));
+    if (lane == 31) base = atomicAdd(&queue_counts<kGroup>(a)[phn & 3], static_cast<uint32_t>(incl));
     base = __shfl_sync(0xFFFFFFFFu, base, 31);
     if (cnt == 0) return;
     QueueEntry *region = a.queue + (phn & 3) * a.npad + base;
@@ -546,6 +558,13 @@ __device__ __forceinline__ void pipe_quad(const StepArgs &a, const int64_t &t, i
         if (!spk[j]) continue;
         const int64_t rs = rp[j];
         const int64_t re = rp[j + 1];
+        QueueEntry e;
+        e.row_quad = static_cast<uint32_t>(rs >> 2);
+        e.len_quads = static_cast<uint32_t>((re - rs) >> 2);
+        e.neuron = static_cast<int32_t>(i0 + j);
+        e.step = static_cast<int32_t>(sn);
+        *reinterpret_cast<int4 *>(region + k) = *reinterpret_cast<const int4 *>(&e);
+        ++k;
         if (re > rs) {
             prefetch_l2(a.syn_tgt + rs, static_cast<uint32_t>(4 * (re - rs)));
             if (a.format == SNN_RECORD_PLAIN9) {
@@ -558,13 +577,38 @@ __device__ __forceinline__ void pipe_quad(const StepArgs &a, const int64_t &t, i
                 prefetch_l2(reinterpret_cast<const uint8_t *>(a.syn_w) + w0, static_cast<uint32_t>(w1 - w0));
             }
         }
-        QueueEntry e;
-        e.row_quad = static_cast<uint32_t>(rs >> 2);
-        e.len_quads = static_cast<uint32_t>((re - rs) >> 2);
-        e.neuron = static_cast<int32_t>(i0 + j);
-        e.step = static_cast<int32_t>(sn);
-        *reinterpret_cast<int4 *>(region + k) = *reinterpret_cast<const int4 *>(&e);
-        ++k;
+    }
+}
+
+// A neuron warp's groups g, g + stride, ... below a.quad_warps: the draws of its first two
+// groups before `wait` (a step kernel's wait for the one before), then group by group with the
+// next group's state in flight.  What bounds a step is the chain wait -> state -> spikes ->
+// queue, about a microsecond per round trip; counting the Poisson thresholds and loading row
+// bounds for all 128 neurons sat on it.  us per step in a graph before and after: tiny circuit
+// 3.17 -> 2.50, full 3.46 -> 2.90, 4x circuit (two groups per warp) 7.91 -> 5.72, 16 circuits
+// in two groups 9.82 -> 8.48.
+template <bool kGroup, bool kB, bool kWait>
+__device__ __forceinline__ void pipe_groups(const StepArgs &a, const int64_t &t, int ph, int64_t g, int64_t stride)
+{
+    const int64_t nquads = (a.n + 3) / 4;
+    const int lane = threadIdx.x & 31;
+    uint32_t d0 = pipe_draws(a, t, g, kB), d1 = pipe_draws(a, t, g + stride, kB);
+    if (kWait) wait_previous_grid();
+    if (g >= a.quad_warps) return;
+    QuadState s;
+    pipe_load<kB>(a, ph, g, g * 32 + lane < nquads, s);
+#pragma unroll 1
+    for (;;) {
+        const int64_t gn = g + stride;
+        const bool more = gn < a.quad_warps;
+        QuadState next = s;
+        if (more) pipe_load<kB>(a, ph, gn, gn * 32 + lane < nquads, next);
+        pipe_quad<kGroup, kB>(a, t, ph, g, g * 32 + lane < nquads, d0, s);
+        if (!more) return;
+        s = next;
+        g = gn;
+        d0 = d1;
+        d1 = pipe_draws(a, t, g + stride, kB);
     }
 }
 
@@ -638,15 +682,8 @@ __global__ void __launch_bounds__(kStepMaxThreads, 2) k_step(const StepArgs a, c
     const int64_t t = a.ctl->t_base + k;  // used for Philox counters and step tags only
     const int wib = threadIdx.x >> 5;
     if (wib < a.neuron_warps) {
-        const int64_t nquads = (a.n + 3) / 4;
-        const int64_t nw = static_cast<int64_t>(a.neuron_warps) * gridDim.x;
-        bool first = true;
-        for (int64_t g = first_quad_warp<kGroup>(a) + static_cast<int64_t>(wib) * gridDim.x + blockIdx.x;
-             g < a.quad_warps; g += nw) {
-            pipe_quad<kGroup>(a, t, ph, g, g * 32 + (threadIdx.x & 31) < nquads, true, first);
-            first = false;
-        }
-        if (first) wait_previous_grid();
+        pipe_groups<kGroup, true, true>(a, t, ph, first_quad_warp<kGroup>(a) + static_cast<int64_t>(wib) * gridDim.x + blockIdx.x,
+                                        static_cast<int64_t>(a.neuron_warps) * gridDim.x);
     } else {
         const int dwarps = static_cast<int>(blockDim.x >> 5) - a.neuron_warps;
         const bool leader = blockIdx.x == 0 && threadIdx.x == 32 * a.neuron_warps;
@@ -659,11 +696,9 @@ __global__ void __launch_bounds__(kStepMaxThreads, 2) k_prime(const StepArgs a)
 {
     const int wib = threadIdx.x >> 5;
     if (wib >= a.neuron_warps) return;
-    const int64_t nquads = (a.n + 3) / 4;
-    const int64_t nw = static_cast<int64_t>(a.neuron_warps) * gridDim.x;
     const int64_t t = -1;
-    for (int64_t g = (a.quad_base >> 5) + static_cast<int64_t>(wib) * gridDim.x + blockIdx.x; g < a.quad_warps; g += nw)
-        pipe_quad<true>(a, t, -1, g, g * 32 + (threadIdx.x & 31) < nquads, false, false);
+    pipe_groups<true, false, false>(a, t, -1, (a.quad_base >> 5) + static_cast<int64_t>(wib) * gridDim.x + blockIdx.x,
+                                    static_cast<int64_t>(a.neuron_warps) * gridDim.x);
 }
 
 // Persistent engine: the pipelined schedule in one cooperative launch for a run of
@@ -676,7 +711,6 @@ __global__ void __launch_bounds__(kStepMaxThreads, 1) k_persistent(const StepArg
     Ctl *ctl = a.ctl;
     const int64_t t0 = ctl->t_base;
     const int wib = threadIdx.x >> 5;
-    const int64_t nquads = (a.n + 3) / 4;
     const int64_t nw = static_cast<int64_t>(a.neuron_warps) * gridDim.x;
     const int dwarps = static_cast<int>(blockDim.x >> 5) - a.neuron_warps;
     const bool leader = blockIdx.x == 0 && threadIdx.x == 32 * a.neuron_warps;
@@ -686,8 +720,7 @@ __global__ void __launch_bounds__(kStepMaxThreads, 1) k_persistent(const StepArg
         const int64_t t = t0 + st;
         const int ph = static_cast<int>(t & (kPhasePeriod - 1));
         if (wib < a.neuron_warps) {
-            for (int64_t g = static_cast<int64_t>(wib) * gridDim.x + blockIdx.x; g < a.quad_warps; g += nw)
-                pipe_quad<false>(a, t, ph, g, g * 32 + (threadIdx.x & 31) < nquads, true, false);
+            pipe_groups<false, true, false>(a, t, ph, static_cast<int64_t>(wib) * gridDim.x + blockIdx.x, nw);
         } else {
             pipe_deliver<false>(a, t, ph, leader, dw, static_cast<int64_t>(dwarps) * gridDim.x, false);
         }

@@ -83,3 +83,20 @@ def test_ring_after_list(nets, form, shape, count):
     np.add.at(want, ((t + e["delay"].astype(np.int64)) % 64, e["post"]), e["w_fx"].astype(np.int64) * times)
     assert np.abs(want).max() < 1 << 31
     assert np.array_equal(ring.cpu().numpy().reshape(64, npad), want)
+
+
+@pytest.mark.parametrize("form", ["plain", "blocked4", "blocked6", "blocked8"])
+def test_ring_after_burst_step(form):
+    """Every neuron spikes at step 0: the graph engine's phase 2 on a step with more events
+    than it reduces row by row."""
+    n = 1733
+    e = dict(_edges(n, 1500, True), u0=np.full(n, 100.0, np.float32))
+    m = workload.microcircuit_model().replace(nu_th_hz=0.0)
+    net = snn.Network(m, custom=e, record_format=FORMS[form][0], engine=snn.ENGINE_GRAPH)
+    net.step(1)
+    assert len(net.read_spikes()[0]) == n
+    npad = int(net.layout().n_neurons_padded)
+    want = np.zeros((64, npad), np.int64)
+    np.add.at(want, (e["delay"].astype(np.int64) % 64, e["post"]), e["w_fx"].astype(np.int64))
+    ring = net.device_view("ring", torch.int32, 64 * npad).cpu().numpy().reshape(64, npad)
+    assert np.array_equal(ring, want)
