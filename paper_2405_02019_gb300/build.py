@@ -19,7 +19,7 @@ BUILD = os.path.join(HERE, "_build")
 ROOT = os.path.dirname(HERE)
 
 SOURCES = ["builder.cpp", "kernels.cu", "blocked.cu", "slices.cu", "resident.cu", "raster.cu", "abi.cu", "noalloc.cu"]
-HEADERS = ["internal.hpp", "philox.cuh", "stream.cuh"]
+HEADERS = ["internal.hpp", "launch.cuh", "philox.cuh", "stream.cuh"]
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 
 

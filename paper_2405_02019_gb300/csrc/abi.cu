@@ -128,10 +128,10 @@ struct HandleScope {
 namespace {
 
 // Phase 2 of graph-engine step t_base + k: blocked records have their own kernel.
-void launch_phase2(const snn_net *net, int k, cudaStream_t st)
+void launch_phase2(const snn_net *net, int k, cudaStream_t st, bool programmatic = false)
 {
-    if (snn::is_blocked(net->format)) snn::launch_deliver_blocked(net->args, nullptr, 0, 0, k, st);
-    else snn::launch_deliver(net->args, k, net->deliver_grid, st);
+    if (snn::is_blocked(net->format)) snn::launch_deliver_blocked(net->args, nullptr, 0, 0, k, st, programmatic);
+    else snn::launch_deliver(net->args, k, net->deliver_grid, st, programmatic);
 }
 
 // Pipelined engine: neuron warps per CTA so that `grid` CTAs cover `quad_warps` groups
@@ -241,6 +241,7 @@ int regroup_queue(snn_net *net, int old_cpg)
 }
 
 // Graph engine: m steps from the device's t_base, every group in turn, then t_base += m.
+// Every kernel but a group's first overlaps its launch with the one before it.
 void enqueue_graph_steps(snn_net *net, int64_t m, cudaStream_t st)
 {
     const size_t G = net->group_args.size();
@@ -248,8 +249,8 @@ void enqueue_graph_steps(snn_net *net, int64_t m, cudaStream_t st)
         const snn::StepArgs &a = G ? net->group_args[g] : net->args;
         const int grid = G ? net->group_grid[g] : net->update_grid;
         for (int64_t k = 0; k < m; ++k) {
-            snn::launch_update(a, static_cast<int>(k), grid, st);
-            launch_phase2(net, static_cast<int>(k), st);
+            snn::launch_update(a, static_cast<int>(k), grid, st, k > 0);
+            launch_phase2(net, static_cast<int>(k), st, true);
         }
         if (g + 1 < G) snn::launch_resync(net->args.ctl, st);
     }
@@ -809,6 +810,8 @@ int snn_build_network(const snn_spec *spec, void *dev_arena, uint64_t arena_byte
         a.rast_t = reinterpret_cast<int32_t *>(A + L.rast_t);
         a.n = net->n;
         a.n_all = net->n;
+        a.quad_warps = static_cast<int32_t>(((net->n + 3) / 4 + 31) / 32);
+        a.mean_row = static_cast<int32_t>(net->n_syn / net->n);
         a.npad = net->npad;
         a.seed = net->circuits[0].seed;  // of the only circuit
         a.rast_cap = static_cast<uint32_t>(L.rast_cap);
@@ -864,7 +867,6 @@ int snn_build_network(const snn_spec *spec, void *dev_arena, uint64_t arena_byte
             a.U2 = reinterpret_cast<float *>(A + L.U2);
             a.R2 = A + L.R2;
             a.queue = reinterpret_cast<snn::QueueEntry *>(A + L.queue);
-            a.quad_warps = static_cast<int32_t>(quad_warps);
             a.qcount = reinterpret_cast<uint32_t *>(A + L.ctl + offsetof(snn::Ctl, qcnt));
             a.queue_cap = net->npad;
             if (snn::prepare_step_kernel(a) != 0) {

@@ -98,7 +98,8 @@ constexpr int kBlockAlign = 32;              // block boundaries are multiples o
 constexpr int kBlockQuad = 4;                // (row, block) segments are whole quads of records
 constexpr int kBlockedThreads = 1024;
 constexpr int kBlockedBinRows = 48;           // delays below this are summed in shared memory (longer: ring reductions)
-constexpr int64_t kBlockedAggregateMin = 64; // fewer senders: reduce straight into the ring
+constexpr int64_t kBlockedAggregateMin = 64; // block-major lists of fewer senders: reduce straight into the ring
+constexpr int64_t kBlockedRowEvents = 1000000; // blocked lists of fewer expected events: row by row (blocked.cu)
 inline int max_target_blocks(int64_t n)
 {
     return static_cast<int>((n + kBlockAvgWidth - 1) / kBlockAvgWidth + n / (kBlockMaxWidth - kBlockAlign) + 2);
@@ -195,7 +196,7 @@ struct StepArgs {
     const uint16_t *blk_seg;      // blocked records: [n][n_blocks + 1] block starts within each row
     const int32_t *blk_off;       // blocked records: block boundaries [n_blocks + 1]
     int32_t n_blocks;
-    int32_t pad4;
+    int32_t mean_row;             // synapses of an average row
     int64_t quad_base;            // first quad the update (or step) launch covers, n its end neuron
     int64_t queue_cap;            // pipelined engine: entries of each queue (a circuit group's neurons)
     uint32_t *mbox;               // resident engine: outboxes [4][n_blocks][kResidentMboxWords]
@@ -298,8 +299,10 @@ bool build_host_network(const snn_spec &spec, const Constants &c, HostNetwork &n
 int resolve_threads(int32_t requested);
 
 // kernels.cu
-void launch_update(const StepArgs &a, int k, int grid, void *stream);
-void launch_deliver(const StepArgs &a, int k, int grid, void *stream);
+// (programmatic: the launch may begin while the previous kernel in the stream still runs; it
+// waits inside)
+void launch_update(const StepArgs &a, int k, int grid, void *stream, bool programmatic = false);
+void launch_deliver(const StepArgs &a, int k, int grid, void *stream, bool programmatic = false);
 void launch_advance(Ctl *ctl, int64_t m, void *stream);
 // circuit groups: the next group starts the same steps where the raster now ends
 void launch_resync(Ctl *ctl, void *stream);
@@ -319,7 +322,8 @@ int step_threads(const StepArgs &a);
 // blocked.cu: one CTA per target block; list == nullptr delivers step t_base + k's
 // spikes from the raster (graph engine), else list[0 .. n) as spikes of step t
 int prepare_blocked_kernel();
-void launch_deliver_blocked(const StepArgs &a, const int32_t *list, int64_t n, int64_t t, int k, void *stream);
+void launch_deliver_blocked(const StepArgs &a, const int32_t *list, int64_t n, int64_t t, int k, void *stream,
+                            bool programmatic = false);
 
 // slices.cu: list[0 .. n) as spikes of step t, on rows with a delay table
 bool slices_pay(const SlicePlan &plan, int64_t n_senders, int64_t events);

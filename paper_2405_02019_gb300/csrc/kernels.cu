@@ -35,6 +35,7 @@
 #include <cuda_runtime.h>
 
 #include "internal.hpp"
+#include "launch.cuh"
 #include "philox.cuh"
 
 namespace snn {
@@ -79,16 +80,6 @@ __device__ __forceinline__ void red_release_add_u32(uint32_t *addr, uint32_t v)
     asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(addr), "r"(v) : "memory");
 }
 
-struct SharedTables {
-    uint64_t thr[SNN_MAX_POPS * kPK];
-};
-
-__device__ __forceinline__ void stage_tables(const StepArgs &a, SharedTables &s)
-{
-    for (int j = threadIdx.x; j < SNN_MAX_POPS * kPK; j += blockDim.x) s.thr[j] = (&a.tables->thresholds[0][0])[j];
-    __syncthreads();
-}
-
 __device__ __forceinline__ int32_t neuron_step(const StepArgs &a, float &u, float &cur, uint32_t &r, int32_t in)
 {
     int32_t spike = 0;
@@ -108,10 +99,89 @@ __device__ __forceinline__ int32_t neuron_step(const StepArgs &a, float &u, floa
     return spike;
 }
 
-// Phase 1 for neurons 4q .. 4q+3 (those below n).  The ring row is read through L2
-// (other SMs add into it between steps).
-__device__ __forceinline__ void update_quad(const StepArgs &a, const SharedTables &s, int64_t t, int64_t q,
-                                            int32_t spk[4])
+__device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes)
+{
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
+}
+
+// Bytes [lo, hi) of an array of records, in whole 16-byte units.
+__device__ __forceinline__ void prefetch_bytes(const void *p, int64_t lo, int64_t hi)
+{
+    lo &= ~int64_t{15};
+    hi = (hi + 15) & ~int64_t{15};
+    prefetch_l2(reinterpret_cast<const uint8_t *>(p) + lo, static_cast<uint32_t>(hi - lo));
+}
+
+// Row [rs, re) of the record store into L2 (of every array the format keeps).
+__device__ __forceinline__ void prefetch_row(const StepArgs &a, int64_t rs, int64_t re)
+{
+    if (re <= rs) return;
+    const int tb = a.format == SNN_RECORD_BLOCKED6 ? 2 : a.format == SNN_RECORD_BLOCKED8 ? 8 : 4;
+    const int wb = a.format == SNN_RECORD_PLAIN9 || a.format == SNN_RECORD_BLOCKED6 ? 4
+                   : a.format == SNN_RECORD_PACKED_BF16                             ? 2
+                   : a.format == SNN_RECORD_PACKED_I8                               ? 1
+                                                                                    : 0;
+    prefetch_bytes(a.syn_tgt, rs * tb, re * tb);
+    if (wb) prefetch_bytes(a.syn_w, rs * wb, re * wb);
+    if (a.format == SNN_RECORD_PLAIN9) prefetch_bytes(a.syn_d, rs, re);
+}
+
+
+// The thalamic counts of four neurons, one byte each, from Philox counter (t, ctr): the
+// first eight thresholds of the first neuron's population are read once and compared with
+// all four words; a count of eight and more goes on from there, and a quad that spans two
+// populations looks each neuron's up.  Not inlined: the step kernel draws in two places.
+__device__ __noinline__ uint32_t draw_quad(uint64_t t, uint64_t ctr, uint64_t seed, uint32_t pops,
+                                           const uint64_t *thresholds)
+{
+    const Block4 rnd = philox4x64_10(t, ctr, 0, 0, seed, kStreamThalamic);
+    const uint64_t *thr = thresholds + (pops & 0xFFu) * kPK;
+    uint32_t T[4] = {0, 0, 0, 0};
+#pragma unroll
+    for (int k = 0; k < 8; k += 2) {
+        const ulonglong2 v2 = __ldg(reinterpret_cast<const ulonglong2 *>(thr + k));
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const uint64_t v = rnd.w[j] >> 1;
+            T[j] += (v >= v2.x ? 1u : 0u) + (v >= v2.y ? 1u : 0u);
+        }
+    }
+    const bool mixed = pops != (pops & 0xFFu) * 0x01010101u;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+        if (!mixed && T[j] < 8u) continue;
+        const uint64_t v = rnd.w[j] >> 1;
+        const uint64_t *own = thresholds + ((pops >> (8 * j)) & 0xFFu) * kPK;
+        uint32_t c = mixed ? 0u : 8u;
+        while (c < static_cast<uint32_t>(kPK) && v >= __ldg(own + c)) ++c;
+        T[j] = c;
+    }
+    return T[0] | (T[1] << 8) | (T[2] << 16) | (T[3] << 24);
+}
+
+// The draws of step t for quad q = 32 g + lane (g: group of 128 neurons), one byte per neuron:
+// the thalamic count, and kDrawValid for a neuron of a circuit (the others are inert).
+// Independent of the dynamics, so a step kernel draws before it waits for the kernel before it.
+constexpr uint32_t kDrawValid = 0x80u;
+__device__ __forceinline__ uint32_t pipe_draws(const StepArgs &a, int64_t t, int64_t g, bool draw)
+{
+    const int64_t i0 = (g * 32 + (threadIdx.x & 31)) * 4;
+    if (g >= a.quad_warps || i0 >= a.n) return 0u;
+    CircuitInfo ci{0, a.n_all, a.seed, 0};
+    if (a.n_circuits > 1) ci = a.circuits[__ldg(a.group_circuit + g)];
+    uint32_t packed = 0;
+    if (draw)
+        packed = draw_quad(static_cast<uint64_t>(t), static_cast<uint64_t>((i0 - ci.base) >> 2), ci.seed,
+                           __ldg(reinterpret_cast<const unsigned int *>(a.pop_id + i0)), a.tables->thresholds[0]);
+    const int64_t left = ci.base + ci.n - i0;  // neurons of the circuit from the quad on
+    return left >= 4 ? packed | kDrawValid * 0x01010101u
+           : left > 0 ? packed | (kDrawValid * 0x01010101u >> (8 * (4 - left)))
+                      : packed;
+}
+
+// Phase 1 for neurons 4q .. 4q+3, from their draws.  The ring row is read through L2 (other
+// SMs add into it between steps).
+__device__ __forceinline__ void update_quad(const StepArgs &a, int64_t t, int64_t q, uint32_t draws, int32_t spk[4])
 {
     const int64_t i0 = q * 4;
     const int64_t slot = t & kDMask;
@@ -121,34 +191,25 @@ __device__ __forceinline__ void update_quad(const StepArgs &a, const SharedTable
     int32_t *wrow = a.ring + slot * a.npad + i0;
     const int4 w4 = __ldcg(reinterpret_cast<const int4 *>(wrow));
     *reinterpret_cast<int4 *>(wrow) = make_int4(0, 0, 0, 0);
-    const CircuitInfo ci = a.circuits[a.group_circuit[i0 >> 7]];
-    const uint32_t pops = *reinterpret_cast<const uint32_t *>(a.pop_id + i0);
-    const Block4 rnd = philox4x64_10(static_cast<uint64_t>(t), static_cast<uint64_t>((i0 - ci.base) >> 2), 0, 0,
-                                     ci.seed, kStreamThalamic);
     float uu[4] = {u4.x, u4.y, u4.z, u4.w};
     float cc[4] = {c4.x, c4.y, c4.z, c4.w};
     const int32_t ww[4] = {w4.x, w4.y, w4.z, w4.w};
     uint32_t rr[4] = {r4 & 0xFFu, (r4 >> 8) & 0xFFu, (r4 >> 16) & 0xFFu, r4 >> 24};
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
-        const int64_t i = i0 + j;
-        if (i < ci.base + ci.n) {
-            const int b = (pops >> (8 * j)) & 0xFF;
-            const uint64_t v = rnd.w[j] >> 1;
-            const uint64_t *thr = s.thr + b * kPK;
-            uint32_t T = 0;
-            while (T < static_cast<uint32_t>(kPK) && v >= thr[T]) ++T;
-            const int32_t in =
-                static_cast<int32_t>(static_cast<uint32_t>(ww[j]) + T * static_cast<uint32_t>(a.w_ext_fx));
-            spk[j] = neuron_step(a, uu[j], cc[j], rr[j], in);
-        }
+        const uint32_t draw = (draws >> (8 * j)) & 0xFFu;
+        if (!(draw & kDrawValid)) continue;
+        const int32_t in =
+            static_cast<int32_t>(static_cast<uint32_t>(ww[j]) + (draw & 0x7Fu) * static_cast<uint32_t>(a.w_ext_fx));
+        spk[j] = neuron_step(a, uu[j], cc[j], rr[j], in);
     }
     *reinterpret_cast<float4 *>(a.U + i0) = make_float4(uu[0], uu[1], uu[2], uu[3]);
     *reinterpret_cast<float4 *>(a.I + i0) = make_float4(cc[0], cc[1], cc[2], cc[3]);
     *reinterpret_cast<uint32_t *>(a.R + i0) = rr[0] | (rr[1] << 8) | (rr[2] << 16) | (rr[3] << 24);
 }
 
-// Warp-collective (every lane must call): append the warp's spikers to the raster.
+// Warp-collective (every lane must call): append the warp's spikers to the raster, and fetch
+// the rows that phase 2 reads next into L2 (their bounds in the append's round trip).
 __device__ __forceinline__ void append_spikes(const StepArgs &a, int64_t t, int64_t i0, const int32_t spk[4])
 {
     const int lane = threadIdx.x & 31;
@@ -161,6 +222,13 @@ __device__ __forceinline__ void append_spikes(const StepArgs &a, int64_t t, int6
     }
     const int total = __shfl_sync(0xFFFFFFFFu, incl, 31);
     if (total == 0) return;
+    int64_t rp[5] = {0, 0, 0, 0, 0};
+    if (cnt != 0) {
+        const longlong2 rpa = __ldg(reinterpret_cast<const longlong2 *>(a.row_ptr + i0));
+        const longlong2 rpb = __ldg(reinterpret_cast<const longlong2 *>(a.row_ptr + i0 + 2));
+        rp[0] = rpa.x; rp[1] = rpa.y; rp[2] = rpb.x; rp[3] = rpb.y;
+        rp[4] = __ldg(a.row_ptr + i0 + 4);
+    }
     uint32_t base = 0;
     if (lane == 31) base = atomicAdd(&a.ctl->cursor, static_cast<uint32_t>(total));
     base = __shfl_sync(0xFFFFFFFFu, base, 31);
@@ -175,6 +243,7 @@ __device__ __forceinline__ void append_spikes(const StepArgs &a, int64_t t, int6
                 atomicOr(&a.ctl->err, kErrRaster);
             }
             ++pos;
+            prefetch_row(a, rp[j], rp[j + 1]);
         }
     }
 }
@@ -282,22 +351,30 @@ __device__ __forceinline__ void deliver_list(const StepArgs &a, int64_t t, const
     else deliver_list_fmt<SNN_RECORD_PLAIN9>(a, t, list, nspk, warp, nwarps);
 }
 
+// Graph engine.  Both kernels start while the kernel before them drains (programmatic
+// launches; t_base as in k_step) and wait for it after the part that does not depend on it.
+// With the rows fetched into L2 by the append and blocked rows reduced by all warps together,
+// a step of the half-scale circuit with BLOCKED8 records went from 8.7 to 7.7 us in a graph and
+// from 12.3 to 8.4 launched one by one.
 __global__ void __launch_bounds__(kUpdateThreads) k_update(const StepArgs a, const int k)
 {
-    __shared__ SharedTables s;
-    stage_tables(a, s);
+    allow_next_grid();
     const int64_t t = a.ctl->t_base + k;
     const int64_t q = a.quad_base + static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+    const uint32_t draws = pipe_draws(a, t, q >> 5, true);
+    wait_previous_grid();
     int32_t spk[4] = {0, 0, 0, 0};
-    if (q * 4 < a.n) update_quad(a, s, t, q, spk);
+    if (q * 4 < a.n) update_quad(a, t, q, draws, spk);
     append_spikes(a, t, q * 4, spk);
 }
 
 __global__ void __launch_bounds__(kDeliverThreads) k_deliver(const StepArgs a, const int k)
 {
+    allow_next_grid();
     const int64_t t = a.ctl->t_base + k;
-    const uint32_t cur = a.ctl->cursor;
-    const uint32_t begin = a.ctl->step_begin[t & 1];
+    wait_previous_grid();
+    const uint32_t cur = __ldcg(&a.ctl->cursor);
+    const uint32_t begin = __ldcg(&a.ctl->step_begin[t & 1]);
     if (blockIdx.x == 0 && threadIdx.x == 0) a.ctl->step_begin[(t + 1) & 1] = cur;
     const uint32_t end = cur < a.rast_cap ? cur : a.rast_cap;
     const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
@@ -380,16 +457,6 @@ __device__ __forceinline__ bool grid_barrier(const StepArgs &a, Ctl *ctl, uint32
 // launch passes in (`ph`).
 // ---------------------------------------------------------------------------
 
-__device__ __forceinline__ void prefetch_l2(const void *p, uint32_t bytes)
-{
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"(bytes) : "memory");
-}
-
-// Waits until the previous kernel of the stream has completed and its writes are
-// visible (a no-op unless this launch was made programmatic).
-__device__ __forceinline__ void wait_previous_grid() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void allow_next_grid() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // A launch of one circuit group (kGroup) takes its queue counts, queue size and first
 // group of 128 neurons from the arguments; a launch over the whole index space uses the
 // control block's counts, npad entries per queue and group 0.  The two are separate
@@ -408,58 +475,6 @@ template <bool kGroup>
 __device__ __forceinline__ int64_t first_quad_warp(const StepArgs &a)
 {
     return kGroup ? (a.quad_base >> 5) : 0;
-}
-
-// The thalamic counts of four neurons, one byte each, from Philox counter (t, ctr): the
-// first eight thresholds of the first neuron's population are read once and compared with
-// all four words; a count of eight and more goes on from there, and a quad that spans two
-// populations looks each neuron's up.  Not inlined: the step kernel draws in two places.
-__device__ __noinline__ uint32_t draw_quad(uint64_t t, uint64_t ctr, uint64_t seed, uint32_t pops,
-                                           const uint64_t *thresholds)
-{
-    const Block4 rnd = philox4x64_10(t, ctr, 0, 0, seed, kStreamThalamic);
-    const uint64_t *thr = thresholds + (pops & 0xFFu) * kPK;
-    uint32_t T[4] = {0, 0, 0, 0};
-#pragma unroll
-    for (int k = 0; k < 8; k += 2) {
-        const ulonglong2 v2 = __ldg(reinterpret_cast<const ulonglong2 *>(thr + k));
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const uint64_t v = rnd.w[j] >> 1;
-            T[j] += (v >= v2.x ? 1u : 0u) + (v >= v2.y ? 1u : 0u);
-        }
-    }
-    const bool mixed = pops != (pops & 0xFFu) * 0x01010101u;
-#pragma unroll
-    for (int j = 0; j < 4; ++j) {
-        if (!mixed && T[j] < 8u) continue;
-        const uint64_t v = rnd.w[j] >> 1;
-        const uint64_t *own = thresholds + ((pops >> (8 * j)) & 0xFFu) * kPK;
-        uint32_t c = mixed ? 0u : 8u;
-        while (c < static_cast<uint32_t>(kPK) && v >= __ldg(own + c)) ++c;
-        T[j] = c;
-    }
-    return T[0] | (T[1] << 8) | (T[2] << 16) | (T[3] << 24);
-}
-
-// The draws of step t for quad q = 32 g + lane (g: group of 128 neurons), one byte per neuron:
-// the thalamic count, and kDrawValid for a neuron of a circuit (the others are inert).
-// Independent of the dynamics, so a step kernel draws before it waits for the kernel before it.
-constexpr uint32_t kDrawValid = 0x80u;
-__device__ __forceinline__ uint32_t pipe_draws(const StepArgs &a, int64_t t, int64_t g, bool draw)
-{
-    const int64_t i0 = (g * 32 + (threadIdx.x & 31)) * 4;
-    if (g >= a.quad_warps || i0 >= a.n) return 0u;
-    CircuitInfo ci{0, a.n_all, a.seed, 0};
-    if (a.n_circuits > 1) ci = a.circuits[__ldg(a.group_circuit + g)];
-    uint32_t packed = 0;
-    if (draw)
-        packed = draw_quad(static_cast<uint64_t>(t), static_cast<uint64_t>((i0 - ci.base) >> 2), ci.seed,
-                           __ldg(reinterpret_cast<const unsigned int *>(a.pop_id + i0)), a.tables->thresholds[0]);
-    const int64_t left = ci.base + ci.n - i0;  // neurons of the circuit from the quad on
-    return left >= 4 ? packed | kDrawValid * 0x01010101u
-           : left > 0 ? packed | (kDrawValid * 0x01010101u >> (8 * (4 - left)))
-                      : packed;
 }
 
 // The dynamic state of a quad, loaded in one round trip.
@@ -565,18 +580,7 @@ __device__ __forceinline__ void pipe_quad(const StepArgs &a, const int64_t &t, i
         e.step = static_cast<int32_t>(sn);
         *reinterpret_cast<int4 *>(region + k) = *reinterpret_cast<const int4 *>(&e);
         ++k;
-        if (re > rs) {
-            prefetch_l2(a.syn_tgt + rs, static_cast<uint32_t>(4 * (re - rs)));
-            if (a.format == SNN_RECORD_PLAIN9) {
-                prefetch_l2(a.syn_w + rs, static_cast<uint32_t>(4 * (re - rs)));
-                const int64_t d0 = rs & ~int64_t{15}, d1 = (re + 15) & ~int64_t{15};
-                prefetch_l2(a.syn_d + d0, static_cast<uint32_t>(d1 - d0));
-            } else {
-                const int64_t bp = a.format == SNN_RECORD_PACKED_I8 ? 1 : 2;
-                const int64_t w0 = (rs * bp) & ~int64_t{15}, w1 = (re * bp + 15) & ~int64_t{15};
-                prefetch_l2(reinterpret_cast<const uint8_t *>(a.syn_w) + w0, static_cast<uint32_t>(w1 - w0));
-            }
-        }
+        prefetch_row(a, rs, re);
     }
 }
 
@@ -744,24 +748,12 @@ int step_grid(int num_sms, int64_t quad_warps)
 
 int step_threads(const StepArgs &a) { return 32 * (a.neuron_warps + a.delivery_warps); }
 
-static size_t step_smem(const StepArgs &) { return 0; }
-
 int prepare_step_kernel(const StepArgs &) { return 0; }
 
 int launch_step(const StepArgs &a, int k, int ph, int grid, void *stream, bool programmatic)
 {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(step_threads(a));
-    cfg.dynamicSmemBytes = step_smem(a);
-    cfg.stream = static_cast<cudaStream_t>(stream);
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = programmatic ? 1 : 0;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (a.group_launch) return static_cast<int>(cudaLaunchKernelEx(&cfg, k_step<true>, a, k, ph));
-    return static_cast<int>(cudaLaunchKernelEx(&cfg, k_step<false>, a, k, ph));
+    return a.group_launch ? launch_after(k_step<true>, grid, step_threads(a), 0, stream, programmatic, a, k, ph)
+                          : launch_after(k_step<false>, grid, step_threads(a), 0, stream, programmatic, a, k, ph);
 }
 
 void launch_prime(const StepArgs &a, int grid, void *stream)
@@ -775,14 +767,14 @@ int update_grid(int64_t n)
     return static_cast<int>((quads + kUpdateThreads - 1) / kUpdateThreads);
 }
 
-void launch_update(const StepArgs &a, int k, int grid, void *stream)
+void launch_update(const StepArgs &a, int k, int grid, void *stream, bool programmatic)
 {
-    k_update<<<grid, kUpdateThreads, 0, static_cast<cudaStream_t>(stream)>>>(a, k);
+    launch_after(k_update, grid, kUpdateThreads, 0, stream, programmatic, a, k);
 }
 
-void launch_deliver(const StepArgs &a, int k, int grid, void *stream)
+void launch_deliver(const StepArgs &a, int k, int grid, void *stream, bool programmatic)
 {
-    k_deliver<<<grid, kDeliverThreads, 0, static_cast<cudaStream_t>(stream)>>>(a, k);
+    launch_after(k_deliver, grid, kDeliverThreads, 0, stream, programmatic, a, k);
 }
 
 void launch_deliver_list(const StepArgs &a, const int32_t *list, int64_t n, int64_t t, int grid, void *stream)
