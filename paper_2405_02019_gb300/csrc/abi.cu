@@ -71,8 +71,13 @@ struct snn_net {
     int persistent_grid = 0;
     int step_grid = 0;
     cudaStream_t capture_stream = nullptr;
-    cudaGraph_t graph = nullptr;
-    cudaGraphExec_t graph_exec = nullptr;
+    // step graphs of steps_per_graph steps and, longest first, of the lengths that a run's
+    // remainder is made of
+    struct StepGraph {
+        int64_t steps;
+        cudaGraphExec_t exec;
+    };
+    std::vector<StepGraph> graphs;
     int64_t t = 0;
     uint32_t device_error = 0;
     // drained raster, ordered by (step, neuron)
@@ -257,23 +262,21 @@ void enqueue_graph_steps(snn_net *net, int64_t m, cudaStream_t st)
     snn::launch_advance(net->args.ctl, m, st);
 }
 
-// Pipelined engine: m step kernels from step t0 (the device's t_base), every circuit
-// group in turn, then t_base += m.  Consecutive kernels of a group overlap their launch
+// Pipelined engine: m step kernels from the device's t_base, every circuit group in turn, then t_base += m.  Consecutive kernels of a group overlap their launch
 // with the previous one (programmatic edges), inside a captured graph and launched one by
 // one alike; a group's first kernel follows the previous group's resync (or the previous
 // run's k_advance, whose t_base it reads before waiting) in plain stream order.
 // One-by-one launches without the edges took 6.2 us per step at pd_full and at pd_tiny,
 // against 3.5 and 3.3 in a graph: a kernel boundary in plain order drains the GPU, and the
 // next kernel's launch and its network, table and Philox work then sit on the chain.
-int enqueue_pipelined_steps(snn_net *net, int64_t m, cudaStream_t st, int64_t t0)
+int enqueue_pipelined_steps(snn_net *net, int64_t m, cudaStream_t st)
 {
     const size_t G = net->group_args.size();
     for (size_t g = 0; g < std::max<size_t>(G, 1); ++g) {
         const snn::StepArgs &a = G ? net->group_args[g] : net->args;
         const int grid = G ? net->group_grid[g] : net->step_grid;
         for (int64_t k = 0; k < m; ++k) {
-            const int ph = static_cast<int>((t0 + k) % snn::kPhasePeriod);
-            const int e = snn::launch_step(a, static_cast<int>(k), ph, grid, st, k > 0);
+            const int e = snn::launch_step(a, static_cast<int>(k), grid, st, k > 0);
             if (e != 0) return fail(SNN_ECUDA, std::string("step launch: ") + cudaGetErrorString(static_cast<cudaError_t>(e)));
         }
         if (g + 1 < G) snn::launch_resync(net->args.ctl, st);
@@ -282,11 +285,11 @@ int enqueue_pipelined_steps(snn_net *net, int64_t m, cudaStream_t st, int64_t t0
     return SNN_OK;
 }
 
-// m steps launched one by one, starting at step t0 (the device counter t_base equals t0).
-int launch_steps_direct(snn_net *net, int64_t m, cudaStream_t st, int64_t t0)
+// m steps launched one by one from the device's t_base.
+int launch_steps_direct(snn_net *net, int64_t m, cudaStream_t st)
 {
     if (net->engine == SNN_ENGINE_PIPELINED) {
-        const int rc = enqueue_pipelined_steps(net, m, st, t0);
+        const int rc = enqueue_pipelined_steps(net, m, st);
         if (rc) return rc;
     } else {
         enqueue_graph_steps(net, m, st);
@@ -329,42 +332,50 @@ int launch_steps_resident(snn_net *net, int64_t n, cudaStream_t st)
     return SNN_OK;
 }
 
-int capture_graph(snn_net *net)
+int capture_steps(snn_net *net, int64_t steps, cudaGraphExec_t *exec)
 {
-    SNN_CUDA_TRY(cudaStreamCreateWithFlags(&net->capture_stream, cudaStreamNonBlocking));
     SNN_CUDA_TRY(cudaStreamBeginCapture(net->capture_stream, cudaStreamCaptureModeThreadLocal));
-    if (net->engine == SNN_ENGINE_PIPELINED) {
-        // replays start on a multiple of the phase period (see snn_step_n)
-        const int rc = enqueue_pipelined_steps(net, net->steps_per_graph, net->capture_stream, 0);
-        if (rc != SNN_OK) {
-            cudaGraph_t g = nullptr;
-            cudaStreamEndCapture(net->capture_stream, &g);
-            if (g) cudaGraphDestroy(g);
-            return rc;
-        }
-    } else {
-        enqueue_graph_steps(net, net->steps_per_graph, net->capture_stream);
-    }
-    cudaError_t launch_err = cudaGetLastError();
+    int rc = SNN_OK;
+    if (net->engine == SNN_ENGINE_PIPELINED) rc = enqueue_pipelined_steps(net, steps, net->capture_stream);
+    else enqueue_graph_steps(net, steps, net->capture_stream);
+    const cudaError_t launch_err = cudaGetLastError();
     cudaGraph_t g = nullptr;
-    cudaError_t end_err = cudaStreamEndCapture(net->capture_stream, &g);
-    if (launch_err != cudaSuccess) return fail(SNN_ECUDA, std::string("capture: ") + cudaGetErrorString(launch_err));
-    if (end_err != cudaSuccess) return fail(SNN_ECUDA, std::string("end capture: ") + cudaGetErrorString(end_err));
-    net->graph = g;
-    SNN_CUDA_TRY(cudaGraphInstantiate(&net->graph_exec, net->graph, 0));
-    return SNN_OK;
+    const cudaError_t end_err = cudaStreamEndCapture(net->capture_stream, &g);
+    if (rc == SNN_OK && launch_err != cudaSuccess) rc = fail(SNN_ECUDA, std::string("capture: ") + cudaGetErrorString(launch_err));
+    if (rc == SNN_OK && end_err != cudaSuccess) rc = fail(SNN_ECUDA, std::string("end capture: ") + cudaGetErrorString(end_err));
+    if (rc == SNN_OK) {
+        const cudaError_t e = cudaGraphInstantiate(exec, g, 0);
+        if (e != cudaSuccess) rc = fail(SNN_ECUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
+    }
+    if (g) cudaGraphDestroy(g);
+    return rc;
 }
 
-// Replaces the captured step graph after a schedule change.
-int recapture(snn_net *net)
+void drop_graphs(snn_net *net)
 {
-    if (net->graph_exec) cudaGraphExecDestroy(net->graph_exec);
-    if (net->graph) cudaGraphDestroy(net->graph);
-    if (net->capture_stream) cudaStreamDestroy(net->capture_stream);
-    net->graph_exec = nullptr;
-    net->graph = nullptr;
-    net->capture_stream = nullptr;
-    return capture_graph(net);
+    for (auto &g : net->graphs) cudaGraphExecDestroy(g.exec);
+    net->graphs.clear();
+}
+
+// The step graphs.  A run of n steps replays the longest graph that fits again and again and
+// launches what is left (fewer than the shortest graph's steps) one by one.  Steps inside a
+// graph take 3.2 (tiny circuit) to 3.5 us, launched one by one 3.6 to 4.0; a replay costs
+// about 5 us at its ends, where launches do not overlap, so lengths are a factor of four
+// apart.
+int capture_graph(snn_net *net)
+{
+    if (!net->capture_stream) SNN_CUDA_TRY(cudaStreamCreateWithFlags(&net->capture_stream, cudaStreamNonBlocking));
+    drop_graphs(net);
+    std::vector<int64_t> lengths{net->steps_per_graph};
+    for (int64_t m : {512, 128, 32, 8})
+        if (m < net->steps_per_graph) lengths.push_back(m);
+    for (int64_t m : lengths) {
+        cudaGraphExec_t exec = nullptr;
+        const int rc = capture_steps(net, m, &exec);
+        if (rc) return rc;
+        net->graphs.push_back({m, exec});
+    }
+    return SNN_OK;
 }
 
 int wait_done(snn_net *net)
@@ -993,21 +1004,11 @@ int snn_step_n(snn_net *net, int64_t n_steps, void *cuda_stream)
                                                           : launch_steps_persistent(net, n_steps, st);
         if (rc) return rc;
     } else {
-        int64_t t = net->t, n = n_steps;
-        if (net->engine == SNN_ENGINE_PIPELINED) {
-            // single steps up to the next multiple of the phase period, where graphs start
-            const int64_t head = std::min<int64_t>(n, (snn::kPhasePeriod - t % snn::kPhasePeriod) % snn::kPhasePeriod);
-            if (head > 0) {
-                const int rc = launch_steps_direct(net, head, st, t);
-                if (rc) return rc;
-                t += head;
-                n -= head;
-            }
-        }
-        for (; n >= net->steps_per_graph; n -= net->steps_per_graph, t += net->steps_per_graph)
-            SNN_CUDA_TRY(cudaGraphLaunch(net->graph_exec, st));
+        int64_t n = n_steps;
+        for (const auto &g : net->graphs)
+            for (; n >= g.steps; n -= g.steps) SNN_CUDA_TRY(cudaGraphLaunch(g.exec, st));
         if (n > 0) {
-            const int rc = launch_steps_direct(net, n, st, t);
+            const int rc = launch_steps_direct(net, n, st);
             if (rc) return rc;
         }
     }
@@ -1068,8 +1069,7 @@ int snn_profile_steps(snn_net *net, int64_t n_steps, void *cuda_stream, double *
             for (int64_t k = 0; k < m; ++k, ++used) {
                 cudaEventRecord(ev[3 * used], st);
                 if (net->engine == SNN_ENGINE_PIPELINED || net->engine == SNN_ENGINE_PERSISTENT) {
-                    const int ph = static_cast<int>((net->t + done + k) % snn::kPhasePeriod);
-                    snn::launch_step(grouped ? net->group_args[g] : net->args, static_cast<int>(k), ph,
+                    snn::launch_step(grouped ? net->group_args[g] : net->args, static_cast<int>(k),
                                      grouped ? net->group_grid[g] : net->step_grid, st);
                     cudaEventRecord(ev[3 * used + 1], st);
                 } else {
@@ -1400,7 +1400,7 @@ int snn_set_schedule(snn_net *net, int32_t grid_ctas, int32_t delivery_warps, in
         return SNN_OK;
     }
     build_groups(net);  // the group arguments copy the schedule
-    return recapture(net);
+    return capture_graph(net);  // replaces the captured step graphs
 }
 
 int snn_set_circuit_groups(snn_net *net, int32_t circuits_per_group)
@@ -1423,7 +1423,7 @@ int snn_set_circuit_groups(snn_net *net, int32_t circuits_per_group)
         }
     }
     build_groups(net);
-    return recapture(net);
+    return capture_graph(net);  // replaces the captured step graphs
 }
 
 int snn_get_circuits(const snn_net *net, int64_t *base, int64_t *n_neurons)
@@ -1477,8 +1477,7 @@ void snn_destroy(snn_net *net)
 {
     if (!net) return;
     if (net->n_snaps > 0) cudaEventSynchronize(net->snap_ev[(net->n_snaps - 1) % snn_net::kSnaps]);
-    if (net->graph_exec) cudaGraphExecDestroy(net->graph_exec);
-    if (net->graph) cudaGraphDestroy(net->graph);
+    drop_graphs(net);
     if (net->capture_stream) cudaStreamDestroy(net->capture_stream);
     for (int k = 0; k < snn_net::kSnaps; ++k)
         if (net->snap_ev[k]) cudaEventDestroy(net->snap_ev[k]);

@@ -311,9 +311,8 @@ int deliver_list_blocks_per_sm();
 int update_grid(int64_t n);  // CTAs of k_update for n neurons
 int persistent_blocks_per_sm(const StepArgs &a);
 int launch_persistent(const StepArgs &a, int64_t n_steps, int grid, void *stream);
-// pipelined: B(t), A(t+1), D(t); ph = t mod 64.  With `programmatic`, the launch may
-// begin while the previous kernel in the stream still runs (it waits inside).
-int launch_step(const StepArgs &a, int k, int ph, int grid, void *stream, bool programmatic = false);
+// pipelined: B(t), A(t+1), D(t) of step t_base + k
+int launch_step(const StepArgs &a, int k, int grid, void *stream, bool programmatic = false);
 void launch_prime(const StepArgs &a, int grid, void *stream);         // pipelined: A(0)
 int prepare_step_kernel(const StepArgs &a);                           // dynamic shared memory opt-in
 int step_grid(int num_sms, int64_t quad_warps);  // default CTAs of the step kernel

@@ -390,7 +390,11 @@ __global__ void __launch_bounds__(kDeliverThreads) k_deliver_list(const StepArgs
     deliver_list(a, t, list, n, spread_warp(), nwarps);
 }
 
-__global__ void k_advance(Ctl *ctl, int64_t m) { ctl->t_base += m; }
+__global__ void k_advance(Ctl *ctl, int64_t m)
+{
+    wait_previous_grid();
+    ctl->t_base += m;
+}
 
 // Circuit groups run the same steps one group after another: the next group's first
 // step appends its spikes from where the raster ends now.
@@ -453,8 +457,7 @@ __device__ __forceinline__ bool grid_barrier(const StepArgs &a, Ctl *ctl, uint32
 // kernel.  A delivery warp loads the step's spike count and the entry of its first
 // item in the same round trip, then the synapses; the warp delivering chunk 0 of spike
 // j records it at raster position base + j, the raster base advancing once per step
-// (Ctl::step_begin[t mod 2]).  Every buffer choice depends on t mod 64 only, which the
-// launch passes in (`ph`).
+// (Ctl::step_begin[t mod 2]).  Every buffer choice depends on t mod 64 only.
 // ---------------------------------------------------------------------------
 
 // A launch of one circuit group (kGroup) takes its queue counts, queue size and first
@@ -680,10 +683,11 @@ __device__ __forceinline__ void pipe_deliver(const StepArgs &a, const int64_t &t
 // t_base is read before waiting on the previous kernel: it only changes in the k_advance
 // that ends a run of steps, and a run's first kernel is not a programmatic launch.
 template <bool kGroup>
-__global__ void __launch_bounds__(kStepMaxThreads, 2) k_step(const StepArgs a, const int k, const int ph)
+__global__ void __launch_bounds__(kStepMaxThreads, 2) k_step(const StepArgs a, const int k)
 {
     allow_next_grid();
-    const int64_t t = a.ctl->t_base + k;  // used for Philox counters and step tags only
+    const int64_t t = a.ctl->t_base + k;
+    const int ph = static_cast<int>(t & (kPhasePeriod - 1));  // every buffer choice depends on this only
     const int wib = threadIdx.x >> 5;
     if (wib < a.neuron_warps) {
         pipe_groups<kGroup, true, true>(a, t, ph, first_quad_warp<kGroup>(a) + static_cast<int64_t>(wib) * gridDim.x + blockIdx.x,
@@ -750,10 +754,10 @@ int step_threads(const StepArgs &a) { return 32 * (a.neuron_warps + a.delivery_w
 
 int prepare_step_kernel(const StepArgs &) { return 0; }
 
-int launch_step(const StepArgs &a, int k, int ph, int grid, void *stream, bool programmatic)
+int launch_step(const StepArgs &a, int k, int grid, void *stream, bool programmatic)
 {
-    return a.group_launch ? launch_after(k_step<true>, grid, step_threads(a), 0, stream, programmatic, a, k, ph)
-                          : launch_after(k_step<false>, grid, step_threads(a), 0, stream, programmatic, a, k, ph);
+    return a.group_launch ? launch_after(k_step<true>, grid, step_threads(a), 0, stream, programmatic, a, k)
+                          : launch_after(k_step<false>, grid, step_threads(a), 0, stream, programmatic, a, k);
 }
 
 void launch_prime(const StepArgs &a, int grid, void *stream)
@@ -789,10 +793,7 @@ int deliver_list_blocks_per_sm()
     return nb > 0 ? nb : 1;
 }
 
-void launch_advance(Ctl *ctl, int64_t m, void *stream)
-{
-    k_advance<<<1, 1, 0, static_cast<cudaStream_t>(stream)>>>(ctl, m);
-}
+void launch_advance(Ctl *ctl, int64_t m, void *stream) { launch_after(k_advance, 1, 1, 0, stream, true, ctl, m); }
 
 void launch_resync(Ctl *ctl, void *stream) { k_resync<<<1, 1, 0, static_cast<cudaStream_t>(stream)>>>(ctl); }
 
