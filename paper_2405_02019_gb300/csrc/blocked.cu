@@ -36,11 +36,11 @@ namespace {
 constexpr int kBlockedStepThreads = 512;
 constexpr int kBlockedRowBatch = 4;  // segments of a row that a warp takes at least (a round of quads)
 
-// Per format: rounds of 32 quads per set (two sets are in flight).
+// Rounds of 32 quads per set (two sets are in flight), and a record's fields.
 template <int FMT>
 struct BlockedForm {
     static constexpr bool wide = FMT == SNN_RECORD_BLOCKED8;
-    static constexpr int rounds = FMT == SNN_RECORD_BLOCKED4 ? 3 : 2;
+    static constexpr int rounds = 2;  // (of 3 BLOCKED4's 64 registers spill: 105 -> 119 us for 7.6e7 events)
     static constexpr int delay_shift = wide ? 16 : kBlockLocalBits;  // local target below
     static constexpr size_t scratch_bytes(int threads) { return sizeof(uint2) * rounds * threads; }
 };

@@ -20,9 +20,9 @@ int launch_after(void (*kernel)(P...), int grid, int threads, size_t smem, void 
     cfg.stream = static_cast<cudaStream_t>(stream);
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = programmatic ? 1 : 0;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = programmatic ? 1 : 0;
     return static_cast<int>(cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...));
 }
 
