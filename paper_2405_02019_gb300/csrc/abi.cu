@@ -846,6 +846,7 @@ int snn_build_network(const snn_spec *spec, void *dev_arena, uint64_t arena_byte
         a.w_ext_fx = net->c.w_ext_fx;
         for (int b = 0; b <= SNN_MAX_POPS; ++b) a.pop_off[b] = tabs.pop_off[b];
         a.n_pops = spec->model.n_pops;
+        a.pop_ranges = spec->n_circuits <= 0 ? 1 : 0;
         a.barrier_timeout_ns = snn::kBarrierTimeoutNs;
         a.barrier_extra = 0;
         // Fault injection for tests of the bounded barrier wait: with SNN_FAULT=barrier_stall

@@ -183,6 +183,7 @@ struct StepArgs {
     QueueEntry *queue;            // pipelined engine: 4 queues, entry j of queue s at queue[s * npad + j]
     int64_t pop_off[SNN_MAX_POPS + 1];  // population offsets (read from the launch arguments)
     int32_t n_pops;
+    int32_t pop_ranges;           // 1: pop_off gives every neuron's population (not for batches)
     int32_t quad_warps;           // pipelined engine: end of the launch's groups of 128 neurons
     uint32_t *qcount;             // pipelined engine: spikes in each of the 4 queues (Ctl::qcnt, or a circuit group's)
     int32_t format;               // SNN_RECORD_*
