@@ -359,15 +359,16 @@ void drop_graphs(snn_net *net)
 
 // The step graphs.  A run of n steps replays the longest graph that fits again and again and
 // launches what is left (fewer than the shortest graph's steps) one by one.  Steps inside a
-// graph take 3.2 (tiny circuit) to 3.5 us, launched one by one 3.6 to 4.0; a replay costs
+// graph take 2.5 (tiny circuit) to 2.9 us, launched one by one 2.9 to 3.3; a replay costs
 // about 5 us at its ends, where launches do not overlap, so lengths are a factor of four
-// apart.
+// apart.  (A graph of 512 steps too made network set-up 2 ms longer for 15 us per thousand
+// steps.)
 int capture_graph(snn_net *net)
 {
     if (!net->capture_stream) SNN_CUDA_TRY(cudaStreamCreateWithFlags(&net->capture_stream, cudaStreamNonBlocking));
     drop_graphs(net);
     std::vector<int64_t> lengths{net->steps_per_graph};
-    for (int64_t m : {512, 128, 32, 8})
+    for (int64_t m : {128, 32, 8})
         if (m < net->steps_per_graph) lengths.push_back(m);
     for (int64_t m : lengths) {
         cudaGraphExec_t exec = nullptr;
@@ -1006,8 +1007,13 @@ int snn_step_n(snn_net *net, int64_t n_steps, void *cuda_stream)
         if (rc) return rc;
     } else {
         int64_t n = n_steps;
-        for (const auto &g : net->graphs)
-            for (; n >= g.steps; n -= g.steps) SNN_CUDA_TRY(cudaGraphLaunch(g.exec, st));
+        // a caller that captures this stream gets the steps as launches (a graph launch cannot
+        // be captured)
+        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+        if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();
+        if (capture == cudaStreamCaptureStatusNone)
+            for (const auto &g : net->graphs)
+                for (; n >= g.steps; n -= g.steps) SNN_CUDA_TRY(cudaGraphLaunch(g.exec, st));
         if (n > 0) {
             const int rc = launch_steps_direct(net, n, st);
             if (rc) return rc;
