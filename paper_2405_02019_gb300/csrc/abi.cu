@@ -824,6 +824,11 @@ int snn_build_network(const snn_spec *spec, void *dev_arena, uint64_t arena_byte
         a.n_all = net->n;
         a.quad_warps = static_cast<int32_t>(((net->n + 3) / 4 + 31) / 32);
         a.mean_row = static_cast<int32_t>(net->n_syn / net->n);
+        int64_t longest = 1;
+        for (int64_t i = 0; i < net->n; ++i) longest = std::max(longest, hn.row_ptr[i + 1] - hn.row_ptr[i]);
+        a.row_windows = static_cast<int32_t>((longest + 32 * snn::kBlockQuad - 1) / (32 * snn::kBlockQuad));
+        a.queue = reinterpret_cast<snn::QueueEntry *>(A + L.queue);
+        a.queue_cap = net->npad;
         a.npad = net->npad;
         a.seed = net->circuits[0].seed;  // of the only circuit
         a.rast_cap = static_cast<uint32_t>(L.rast_cap);
@@ -879,7 +884,6 @@ int snn_build_network(const snn_spec *spec, void *dev_arena, uint64_t arena_byte
             a.delivery_warps = net->step_grid > net->num_sms ? snn::kStepDeliverWarps / 2 : snn::kStepDeliverWarps;
             a.U2 = reinterpret_cast<float *>(A + L.U2);
             a.R2 = A + L.R2;
-            a.queue = reinterpret_cast<snn::QueueEntry *>(A + L.queue);
             a.qcount = reinterpret_cast<uint32_t *>(A + L.ctl + offsetof(snn::Ctl, qcnt));
             a.queue_cap = net->npad;
             if (snn::prepare_step_kernel(a) != 0) {

@@ -13,14 +13,15 @@
 // read-modify-write.  Longer delays (one microcircuit event in 1e5) go straight to the ring
 // as reductions; they land in other ring rows than the plain adds.  Integer addition makes
 // every order give the same ring.
-// Few events (kBlockedRowEvents; nearly every step of a simulation) are not worth clearing
-// and adding the sums: then all warps of the launch share the (sender, block) segments, a few
-// consecutive ones of a row each, and every record is a reduction into the ring.
-// Measured (CUDA events, a list of 20,480 full-scale senders, 7.6e7 events): BLOCKED8 186 ->
-// 130-134 us, 4.8 TB/s of its own bytes where the measured copy moves 6.8.  Before, the CTA staged
-// 2,048 senders at a time between barriers, so the record reads drained two or three times
-// per pass.  At 2,048 senders of the half-scale circuit BLOCKED4 stays at 22 us: launch,
-// list -> bounds -> records -> ring is one chain of round trips there.
+// Few events (nearly every step of a simulation) are not worth clearing and adding the sums:
+// below kBlockedRowEvents, and while no warp gets more than two windows, all warps of the
+// launch share the rows, a window of 32 consecutive quads at a time, and every record is a
+// reduction into the ring.
+// Measured, 20,480 senders (7.6e7 events): BLOCKED8 at full scale 181 -> 128 us, 4.8 TB/s of
+// its own bytes where a copy moves 6.8; BLOCKED4 and 6 of the half-scale circuit 162 -> 107
+// and 192 -> 169 us.  Before, the CTA staged 2,048 senders at a time between barriers, so the
+// record reads drained two or three times per pass.  Short lists are one chain of round trips,
+// list -> bounds -> records -> ring: BLOCKED4 at 2,048 senders 21.5 -> 20.6 us, at 512 10.3 -> 12.2.
 #include <cuda_runtime.h>
 
 #include "internal.hpp"
@@ -34,7 +35,11 @@ namespace {
 // Threads per CTA: all that fit for a given list; in the step loop half, which leaves the
 // next update kernel room to start beside this one.
 constexpr int kBlockedStepThreads = 512;
-constexpr int kBlockedRowBatch = 4;  // segments of a row that a warp takes at least (a round of quads)
+// Clearing and adding the bins is what a short list pays for: fewer delays are binned below
+// kBlockedLongList senders (512 full-scale senders with BLOCKED8: 14.3 us with 48 rows, 13.5 with
+// 33; at 2,048 both take 23.5).
+constexpr int64_t kBlockedLongList = 2048;
+constexpr int kBlockedShortRows = 33;
 
 // Rounds of 32 quads per set (two sets are in flight), and a record's fields.
 template <int FMT>
@@ -109,7 +114,6 @@ struct BlockedSource {
     using Form = BlockedForm<FMT>;
     static constexpr int kRounds = Form::rounds;
     static constexpr bool kFlags = false;
-    static constexpr uint32_t kLimit = static_cast<uint32_t>(kBlockedBinRows) << Form::delay_shift;
     struct Raw {
         int64_t row;
         uint16_t o0, o1;
@@ -123,6 +127,8 @@ struct BlockedSource {
     uint32_t bins;  // shared address
     int64_t t;
     int32_t base;
+    int32_t stride;  // of the bins
+    uint32_t limit;  // records from here on have a delay that is not binned
     int p;
 
     __device__ __forceinline__ int32_t sender(int64_t j) const { return __ldcg(list + j); }
@@ -168,8 +174,8 @@ struct BlockedSource {
     __device__ __forceinline__ void near(uint32_t rec, int32_t w) const
     {
         const uint32_t d = rec >> Form::delay_shift;
-        const uint32_t i = rec - d * ((1u << Form::delay_shift) - kBlockMaxWidth);
-        add_shared_if(bins + 4 * i, w, rec, kLimit);
+        const uint32_t i = rec - d * ((1u << Form::delay_shift) - static_cast<uint32_t>(stride));
+        add_shared_if(bins + 4 * i, w, rec, limit);
     }
     __device__ __forceinline__ void add(const Set &s) const
     {
@@ -185,7 +191,7 @@ struct BlockedSource {
                 longest = max(longest, rec[e]);
             }
         }
-        if (longest < kLimit) return;
+        if (longest < limit) return;
 #pragma unroll
         for (int k = 0; k < kRounds; ++k) {
             uint32_t rec[4];
@@ -193,75 +199,69 @@ struct BlockedSource {
             blocked_quad<FMT>(s.va[k], s.vb[k], rec, w);
 #pragma unroll
             for (int e = 0; e < 4; ++e)
-                if (w[e] != 0 && rec[e] >= kLimit) reduce_record<FMT>(a, t, base, rec[e], w[e]);
+                if (w[e] != 0 && rec[e] >= limit) reduce_record<FMT>(a, t, base, rec[e], w[e]);
         }
     }
 };
 
-// All blocks' segments of a list's senders: segment j is block j mod n_blocks of sender
-// j div n_blocks, so that consecutive lanes hold consecutive segments of one row.
+// Few events: a warp takes 32 consecutive quads of one row.  Which block a quad belongs to
+// comes from the row's block table, read alongside the quads: each block that starts inside
+// the window marks its first quad, and a lane's block is the last one at or before it.
+// `offs`: the block boundaries, in shared memory; `scratch`: the warp's 32 words.
 template <int FMT>
-struct BlockedRowSource {
-    static constexpr int kRounds = 1;
-    static constexpr bool kFlags = true;  // a unit's flags: the first target of its block
-    struct Raw {
-        int64_t row;
-        int32_t base;
-        uint16_t o0, o1;
-    };
-    struct Set {
-        uint4 va, vb;
-        int32_t base;
-    };
-
-    const StepArgs &a;
-    const int32_t *list;
-    int64_t t;
-
-    __device__ __forceinline__ int32_t sender(int64_t j) const
-    {
-        return __ldcg(list + static_cast<uint32_t>(j) / static_cast<uint32_t>(a.n_blocks));
-    }
-    __device__ __forceinline__ Raw raw(int64_t j, int32_t s) const
-    {
-        const uint32_t p = static_cast<uint32_t>(j) % static_cast<uint32_t>(a.n_blocks);
-        const uint16_t *sg = a.blk_seg + static_cast<int64_t>(s) * (a.n_blocks + 1) + p;
-        return Raw{__ldg(a.row_ptr + s), __ldg(a.blk_off + p), __ldg(sg), __ldg(sg + 1)};
-    }
-    __device__ __forceinline__ Segment segment(const Raw &r) const
-    {
-        return Segment{static_cast<uint32_t>((r.row + r.o0) / kBlockQuad), (r.o1 - r.o0) / kBlockQuad,
-                       static_cast<uint32_t>(r.base)};
-    }
-    __device__ __forceinline__ void load(const StreamUnit (&u)[1], Set &s) const
-    {
-        s.va = make_uint4(0, 0, 0, 0);
-        s.vb = make_uint4(0, 0, 0, 0);
-        s.base = static_cast<int32_t>(u[0].flags);
-        if (!u[0].ok) return;
+__device__ __forceinline__ void blocked_row_window(const StepArgs &a, int64_t t, uint32_t row_quad, uint32_t len,
+                                                   int32_t s, uint32_t w0, const int32_t *offs, int32_t *scratch)
+{
+    constexpr int kPer = 5;  // the table of up to 160 blocks in one round trip
+    const int lane = threadIdx.x & 31;
+    const bool ok = w0 + lane < len;
+    uint4 va = make_uint4(0, 0, 0, 0), vb = va;
+    if (ok) {
+        const uint64_t q = static_cast<uint64_t>(row_quad) + w0 + lane;
         const uint4 *q16 = reinterpret_cast<const uint4 *>(a.blk_rec);
-        const uint64_t q = u[0].index;
         if (FMT == SNN_RECORD_BLOCKED8) {
-            s.va = __ldcs(q16 + 2 * q);
-            s.vb = __ldcs(q16 + 2 * q + 1);
+            va = __ldcs(q16 + 2 * q);
+            vb = __ldcs(q16 + 2 * q + 1);
         } else if (FMT == SNN_RECORD_BLOCKED4) {
-            s.va = __ldcs(q16 + q);
+            va = __ldcs(q16 + q);
         } else {
             const uint2 r = __ldcs(reinterpret_cast<const uint2 *>(a.blk_rec) + q);
-            s.va = make_uint4(r.x, r.y, 0, 0);
-            s.vb = __ldcs(reinterpret_cast<const uint4 *>(a.syn_w) + q);
+            va = make_uint4(r.x, r.y, 0, 0);
+            vb = __ldcs(reinterpret_cast<const uint4 *>(a.syn_w) + q);
         }
     }
-    __device__ __forceinline__ void add(const Set &s) const
-    {
-        uint32_t rec[4];
-        int32_t w[4];
-        blocked_quad<FMT>(s.va, s.vb, rec, w);
+    const uint16_t *sg = a.blk_seg + static_cast<int64_t>(s) * (a.n_blocks + 1);
+    __syncwarp();
+    scratch[lane] = -1;
+    __syncwarp();
+    int before = 0;  // blocks that start at or before the window
+    for (int b0 = 0; b0 < a.n_blocks; b0 += 32 * kPer) {
+        uint32_t st[kPer];
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-            if (w[e] != 0) reduce_record<FMT>(a, t, s.base, rec[e], w[e]);
+        for (int i = 0; i < kPer; ++i)
+            st[i] = b0 + lane + 32 * i < a.n_blocks ? __ldg(sg + b0 + lane + 32 * i) / kBlockQuad : 0xFFFFFFFFu;
+#pragma unroll
+        for (int i = 0; i < kPer; ++i) {
+            before += __popc(__ballot_sync(0xFFFFFFFFu, st[i] <= w0));
+            if (st[i] > w0 && st[i] < w0 + 32) atomicMax(scratch + (st[i] - w0), b0 + lane + 32 * i);
+        }
     }
-};
+    __syncwarp();
+    int b = max(scratch[lane], before - 1);  // empty blocks start where the next one does: the last wins
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xFFFFFFFFu, b, o);
+        if (lane >= o) b = max(b, y);
+    }
+    if (!ok) return;
+    uint32_t rec[4];
+    int32_t w[4];
+    blocked_quad<FMT>(va, vb, rec, w);
+    const int32_t base = offs[b];
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+        if (w[e] != 0) reduce_record<FMT>(a, t, base, rec[e], w[e]);
+}
 
 template <int FMT, int kThreads>
 __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
@@ -270,53 +270,88 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
     using Form = BlockedForm<FMT>;
     extern __shared__ int4 smem4[];
     const uint32_t bins = shared_address(smem4);
+    int32_t *bins_i = reinterpret_cast<int32_t *>(smem4);  // with few events: the block boundaries
     const int tid = threadIdx.x, warp = tid >> 5;
     uint2 *scratch = reinterpret_cast<uint2 *>(reinterpret_cast<uint8_t *>(smem4) + kBlockedBinBytes) + 32 * Form::rounds * warp;
 
     int64_t t;
     const int32_t *spk;
     int64_t nspk;
+    // consecutive warps on consecutive CTAs, so that few windows spread over all SMs
+    const int64_t gw = static_cast<int64_t>(warp) * gridDim.x + blockIdx.x;
+    const int64_t warps = static_cast<int64_t>(kThreads / 32) * gridDim.x;
+    int4 first = make_int4(0, 0, 0, -1);
+    // (the block boundaries of the row by row path fit the bins' memory)
+    bool rows = a.n_blocks <= kBlockedBinRows * kBlockMaxWidth;
+    if (rows && list == nullptr)
+        for (int j = tid; j < a.n_blocks; j += kThreads) bins_i[j] = __ldg(a.blk_off + j);
     if (list != nullptr) {
         t = t_list;
         spk = list;
         nspk = n_list;
     } else {
-        // graph engine: the spikes step t appended to the raster (t_base as in k_step)
+        // graph engine: the spikes step t appended to the raster (t_base as in k_step), and the
+        // entry of this warp's first window in the same round trip
         allow_next_grid();
         t = a.ctl->t_base + k;
+        const int64_t j0 = gw / a.row_windows;
         wait_previous_grid();
         const uint32_t cur = __ldcg(&a.ctl->cursor);
         const uint32_t begin = __ldcg(&a.ctl->step_begin[t & 1]);
+        if (j0 < a.queue_cap) first = __ldcg(reinterpret_cast<const int4 *>(a.queue + (t & 1) * a.npad + j0));
         if (blockIdx.x == 0 && threadIdx.x == 0) a.ctl->step_begin[(t + 1) & 1] = cur;
         const uint32_t end = cur < a.rast_cap ? cur : a.rast_cap;
         spk = a.rast_nrn + begin;
         nspk = end > begin ? static_cast<int64_t>(end - begin) : 0;
     }
     if (nspk == 0) return;
-    if (nspk * a.mean_row < kBlockedRowEvents && nspk * a.n_blocks < (int64_t{1} << 31)) {
-        // consecutive warps on consecutive CTAs, so that few segments spread over all SMs
-        const BlockedRowSource<FMT> src{a, spk, t};
-        WarpStream<BlockedRowSource<FMT>>(src, nspk * a.n_blocks, warp * gridDim.x + blockIdx.x,
-                                          kThreads / 32 * gridDim.x, scratch, kBlockedRowBatch).run();
+    rows = rows && nspk * a.mean_row < kBlockedRowEvents && nspk * a.row_windows <= 2 * warps;
+    if (rows) {
+        if (list != nullptr)
+            for (int j = tid; j < a.n_blocks; j += kThreads) bins_i[j] = __ldg(a.blk_off + j);
+        __syncthreads();
+        for (int64_t it = gw; it < nspk * a.row_windows; it += warps) {
+            const int64_t j = it / a.row_windows;
+            const uint32_t w0 = static_cast<uint32_t>(it - j * a.row_windows) * 32;
+            uint32_t row_quad, len;
+            int32_t s;
+            if (list != nullptr) {
+                s = __ldcg(spk + j);
+                const int64_t rs = __ldg(a.row_ptr + s);
+                row_quad = static_cast<uint32_t>(rs / kBlockQuad);
+                len = static_cast<uint32_t>((__ldg(a.row_ptr + s + 1) - rs) / kBlockQuad);
+            } else {
+                const int4 e = it == gw ? first : __ldcg(reinterpret_cast<const int4 *>(a.queue + (t & 1) * a.npad + j));
+                row_quad = static_cast<uint32_t>(e.x);
+                len = static_cast<uint32_t>(e.y);
+                s = e.z;
+            }
+            if (w0 < len)
+                blocked_row_window<FMT>(a, t, row_quad, len, s, w0, bins_i, reinterpret_cast<int32_t *>(scratch));
+        }
         return;
     }
 
     const int p = blockIdx.x;
     const int32_t base = a.blk_off[p];
-    const int32_t width = a.blk_off[p + 1] - base;
-    const BlockedSource<FMT> src{a, spk, bins, t, base, p};
+    const int32_t stride = BlockedForm<FMT>::wide ? kBlockMaxWidth : (a.blk_off[p + 1] - base + 3) & ~3;
+    // fewer bins to clear and add for a short list
+    const int bin_rows = nspk < kBlockedLongList ? kBlockedShortRows : kBlockedBinRows;
+    const uint32_t limit = static_cast<uint32_t>(bin_rows) << BlockedForm<FMT>::delay_shift;
+    const BlockedSource<FMT> src{a, spk, bins, t, base, stride, limit, p};
     WarpStream<BlockedSource<FMT>> stream(src, nspk, warp, kThreads / 32, scratch);
-    for (int j = tid; j < kBlockedBinRows * kBlockMaxWidth / 4; j += kThreads) smem4[j] = make_int4(0, 0, 0, 0);
+    if (list == nullptr) __syncthreads();  // the block boundaries are written before they are cleared
+    for (int j = tid; j < bin_rows * stride / 4; j += kThreads) smem4[j] = make_int4(0, 0, 0, 0);
     __syncthreads();
     stream.run();
     __syncthreads();
     // add the sums of the binned delays to their ring rows; width is a multiple
     // of 4 except for the last block, whose extra columns lie inside the padded ring row
-    const int w4 = (width + 3) >> 2;
-    for (int q = tid; q < (kBlockedBinRows - 1) * w4; q += kThreads) {
+    const int w4 = (a.blk_off[p + 1] - base + 3) >> 2;
+    for (int q = tid; q < (bin_rows - 1) * w4; q += kThreads) {
         const int d = 1 + q / w4;
         const int c4 = q - (d - 1) * w4;
-        const int4 v = smem4[(d * kBlockMaxWidth) / 4 + c4];
+        const int4 v = smem4[(d * stride) / 4 + c4];
         if ((v.x | v.y | v.z | v.w) == 0) continue;
         int4 *dst = reinterpret_cast<int4 *>(a.ring + ((t + d) & kDMask) * a.npad + base) + c4;
         int4 o = __ldcg(dst);

@@ -99,7 +99,9 @@ constexpr int kBlockQuad = 4;                // (row, block) segments are whole 
 constexpr int kBlockedThreads = 1024;
 constexpr int kBlockedBinRows = 48;           // delays below this are summed in shared memory (longer: ring reductions)
 constexpr int64_t kBlockedAggregateMin = 64; // block-major lists of fewer senders: reduce straight into the ring
-constexpr int64_t kBlockedRowEvents = 1000000; // blocked lists of fewer expected events: row by row (blocked.cu)
+// Blocked lists of fewer expected events go row by row.  64 senders of the half-scale circuit
+// (2.4e5 events) take as long as any launch either way; 256 (9.4e5) 12.3 us row by row, 9.0 summed.
+constexpr int64_t kBlockedRowEvents = 300000;
 inline int max_target_blocks(int64_t n)
 {
     return static_cast<int>((n + kBlockAvgWidth - 1) / kBlockAvgWidth + n / (kBlockMaxWidth - kBlockAlign) + 2);
@@ -180,7 +182,7 @@ struct StepArgs {
     int32_t neuron_warps;         // pipelined engine: neuron warps per CTA
     float *U2;                    // pipelined engine: second U / R buffers (state after A(s) in buffer s mod 2)
     uint8_t *R2;
-    QueueEntry *queue;            // pipelined engine: 4 queues, entry j of queue s at queue[s * npad + j]
+    QueueEntry *queue;            // 4 queues, entry j of queue s at queue[s * npad + j] (graph engine: 2, by step parity)
     int64_t pop_off[SNN_MAX_POPS + 1];  // population offsets (read from the launch arguments)
     int32_t n_pops;
     int32_t pop_ranges;           // 1: pop_off gives every neuron's population (not for batches)
@@ -198,6 +200,8 @@ struct StepArgs {
     const int32_t *blk_off;       // blocked records: block boundaries [n_blocks + 1]
     int32_t n_blocks;
     int32_t mean_row;             // synapses of an average row
+    int32_t row_windows;          // blocked records: windows of 32 quads in the longest row
+    int32_t pad4;
     int64_t quad_base;            // first quad the update (or step) launch covers, n its end neuron
     int64_t queue_cap;            // pipelined engine: entries of each queue (a circuit group's neurons)
     uint32_t *mbox;               // resident engine: outboxes [4][n_blocks][kResidentMboxWords]

@@ -208,9 +208,11 @@ __device__ __forceinline__ void update_quad(const StepArgs &a, int64_t t, int64_
     *reinterpret_cast<uint32_t *>(a.R + i0) = rr[0] | (rr[1] << 8) | (rr[2] << 16) | (rr[3] << 24);
 }
 
-// Warp-collective (every lane must call): append the warp's spikers to the raster, and fetch
-// the rows that phase 2 reads next into L2 (their bounds in the append's round trip).
-__device__ __forceinline__ void append_spikes(const StepArgs &a, int64_t t, int64_t i0, const int32_t spk[4])
+// Warp-collective (every lane must call): append the warp's spikers to the raster, whose
+// entries of this step start at `begin`, and to the step's list of rows (StepArgs::queue, by
+// the step's parity), and fetch those rows into L2 for phase 2.
+__device__ __forceinline__ void append_spikes(const StepArgs &a, int64_t t, int64_t i0, uint32_t begin,
+                                              const int32_t spk[4])
 {
     const int lane = threadIdx.x & 31;
     const int cnt = spk[0] + spk[1] + spk[2] + spk[3];
@@ -241,6 +243,14 @@ __device__ __forceinline__ void append_spikes(const StepArgs &a, int64_t t, int6
                 a.rast_t[pos] = static_cast<int32_t>(t);
             } else {
                 atomicOr(&a.ctl->err, kErrRaster);
+            }
+            if (pos - begin < static_cast<uint32_t>(a.queue_cap)) {
+                QueueEntry e;
+                e.row_quad = static_cast<uint32_t>(rp[j] >> 2);
+                e.len_quads = static_cast<uint32_t>((rp[j + 1] - rp[j]) >> 2);
+                e.neuron = static_cast<int32_t>(i0 + j);
+                e.step = static_cast<int32_t>(t);
+                *reinterpret_cast<int4 *>(a.queue + (t & 1) * a.npad + (pos - begin)) = *reinterpret_cast<const int4 *>(&e);
             }
             ++pos;
             prefetch_row(a, rp[j], rp[j + 1]);
@@ -353,9 +363,10 @@ __device__ __forceinline__ void deliver_list(const StepArgs &a, int64_t t, const
 
 // Graph engine.  Both kernels start while the kernel before them drains (programmatic
 // launches; t_base as in k_step) and wait for it after the part that does not depend on it.
-// With the rows fetched into L2 by the append and blocked rows reduced by all warps together,
-// a step of the half-scale circuit with BLOCKED8 records went from 8.7 to 7.7 us in a graph and
-// from 12.3 to 8.4 launched one by one.
+// A step is a chain of round trips of about 0.7 us: state -> append -> count and row entry ->
+// records -> ring.  A step of the half-scale circuit with BLOCKED8 records took 9.8 us in a
+// graph (14.2 launched one by one); overlapping launches, rows fetched into L2 by the append
+// and all warps sharing few events 7.7; the step's own list of rows, read with the count, 5.8.
 __global__ void __launch_bounds__(kUpdateThreads) k_update(const StepArgs a, const int k)
 {
     allow_next_grid();
@@ -363,23 +374,51 @@ __global__ void __launch_bounds__(kUpdateThreads) k_update(const StepArgs a, con
     const int64_t q = a.quad_base + static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
     const uint32_t draws = pipe_draws(a, t, q >> 5, true);
     wait_previous_grid();
+    const uint32_t begin = __ldcg(&a.ctl->step_begin[t & 1]);
     int32_t spk[4] = {0, 0, 0, 0};
     if (q * 4 < a.n) update_quad(a, t, q, draws, spk);
-    append_spikes(a, t, q * 4, spk);
+    append_spikes(a, t, q * 4, begin, spk);
+}
+
+// Delivery of the step's rows: items as in deliver_list, with the entry of a warp's first item
+// read in the count's round trip.
+template <int FMT>
+__device__ __forceinline__ void deliver_rows_fmt(const StepArgs &a, int64_t t, int64_t nspk, int64_t warp,
+                                                 int64_t nwarps, int4 first)
+{
+    const QueueEntry *rows = a.queue + (t & 1) * a.npad;
+    const int64_t cpr = a.chunks_per_row;
+    const int64_t ipj = items_per_spike(cpr, nspk, nwarps);
+    const int64_t per = (cpr + ipj - 1) / ipj;
+    for (int64_t it = warp; it < nspk * ipj; it += nwarps) {
+        const int64_t j = it / ipj, part = it - j * ipj;
+        const int4 raw = it == warp && ipj == cpr ? first : __ldcg(reinterpret_cast<const int4 *>(rows + j));
+        const int64_t rs = static_cast<int64_t>(static_cast<uint32_t>(raw.x)) * 4;
+        const int64_t re = rs + static_cast<int64_t>(static_cast<uint32_t>(raw.y)) * 4;
+        const int src = FMT == SNN_RECORD_PACKED_I8 ? __ldg(a.pop_id + raw.z) : 0;
+        for (int64_t c = part * per, off = rs + c * kChunk; c < (part + 1) * per && off < re; ++c, off += kChunk)
+            deliver_chunk<FMT>(a, t, off, re, src);
+    }
 }
 
 __global__ void __launch_bounds__(kDeliverThreads) k_deliver(const StepArgs a, const int k)
 {
     allow_next_grid();
     const int64_t t = a.ctl->t_base + k;
+    const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
+    const int64_t warp = spread_warp();
+    const int64_t j0 = warp / a.chunks_per_row;
     wait_previous_grid();
     const uint32_t cur = __ldcg(&a.ctl->cursor);
     const uint32_t begin = __ldcg(&a.ctl->step_begin[t & 1]);
+    const int4 first = j0 < a.queue_cap ? __ldcg(reinterpret_cast<const int4 *>(a.queue + (t & 1) * a.npad + j0))
+                                        : make_int4(0, 0, 0, 0);
     if (blockIdx.x == 0 && threadIdx.x == 0) a.ctl->step_begin[(t + 1) & 1] = cur;
     const uint32_t end = cur < a.rast_cap ? cur : a.rast_cap;
-    const int64_t nwarps = (static_cast<int64_t>(gridDim.x) * blockDim.x) >> 5;
     const int64_t nspk = end > begin ? static_cast<int64_t>(end - begin) : 0;
-    deliver_list(a, t, a.rast_nrn + begin, nspk, spread_warp(), nwarps);
+    if (a.format == SNN_RECORD_PACKED_I8) deliver_rows_fmt<SNN_RECORD_PACKED_I8>(a, t, nspk, warp, nwarps, first);
+    else if (a.format == SNN_RECORD_PACKED_BF16) deliver_rows_fmt<SNN_RECORD_PACKED_BF16>(a, t, nspk, warp, nwarps, first);
+    else deliver_rows_fmt<SNN_RECORD_PLAIN9>(a, t, nspk, warp, nwarps, first);
 }
 
 // Phase 2 alone for a caller-given list of senders (measurement and tests).

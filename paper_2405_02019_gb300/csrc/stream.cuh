@@ -170,14 +170,12 @@ struct WarpStream {
         s_next = fetch();
     }
 
-    // (batches of at least `least` segments, where fewer would leave most of a round empty)
-    __device__ __forceinline__ WarpStream(const Source &source, int64_t count, int warp, int warps, uint2 *scr,
-                                          int least = 1)
+    __device__ __forceinline__ WarpStream(const Source &source, int64_t count, int warp, int warps, uint2 *scr)
         : src(source), n(count), scratch(scr)
     {
         // passes of all warps over the list, each as even as its batches of at most 32 allow
         const int64_t passes = (n + 32 * warps - 1) / (32 * warps);
-        size = max(least, static_cast<int32_t>((n + warps * passes - 1) / (warps * passes)));
+        size = static_cast<int32_t>((n + warps * passes - 1) / (warps * passes));
         step = static_cast<int64_t>(size) * warps;
         at = static_cast<int64_t>(size) * warp + (threadIdx.x & 31);
         s_next = fetch();
