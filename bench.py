@@ -1,7 +1,8 @@
 """Benchmark of the full-scale Potjans-Diesmann microcircuit step loop on GB300.
 
 One bench step = 1,024 simulation steps of 0.1 ms (102.4 ms of biological time: one
-launch of the resident engine, by default, or one CUDA-graph replay) of the full microcircuit (77,169 neurons, 284,811,022 synapses,
+CUDA-graph replay of the pipelined engine, by default, or one launch of the resident engine)
+of the full microcircuit (77,169 neurons, 284,811,022 synapses,
 seed 1 + rank), so the default --steps 100 covers the paper's 10 s runs (§4).  Prints
 one JSON line.
 
@@ -68,23 +69,27 @@ def _kernel_sources_hash(files=("kernels.cu", "internal.hpp")) -> str:
 
 
 # the sources each recorded kernel is built from
-_RESIDENT_KERNELS = ("k_resident", "k_deliver_regions")
+_SOURCES = {
+    "k_step": ("kernels.cu", "launch.cuh", "internal.hpp"),
+    "k_deliver_slices": ("slices.cu", "stream.cuh", "internal.hpp"),
+    "k_deliver_blocked": ("blocked.cu", "stream.cuh", "internal.hpp"),
+    "k_resident": ("resident.cu", "stream.cuh", "internal.hpp"),
+    "k_deliver_regions": ("resident.cu", "stream.cuh", "internal.hpp"),
+}
 
 
 def _recorded_traffic(kernel: str):
     """DRAM bytes per launch from the committed ncu record, only if the kernel's sources
-    are unchanged since it was taken."""
+    are unchanged since it was taken.  A record may be of one variant of a kernel
+    (k_deliver_blocked_8)."""
     p = os.path.join(ROOT, "profiles", "traffic.json")
     if not os.path.exists(p):
         return None
-    d = json.load(open(p))
-    if kernel in _RESIDENT_KERNELS:
-        valid = d.get("resident_sha256_16") == _kernel_sources_hash(("resident.cu", "internal.hpp"))
-    else:
-        valid = d.get("kernels_sha256_16") == _kernel_sources_hash()
-    if not valid or kernel not in d:
+    rec = json.load(open(p)).get(kernel)
+    src = next((f for k, f in _SOURCES.items() if kernel.startswith(k)), None)
+    if rec is None or src is None or rec.get("sources_sha256_16") != _kernel_sources_hash(src):
         return None
-    return d[kernel].get("dram_bytes_per_launch")
+    return rec.get("dram_bytes_per_launch")
 
 
 def thalamic_events_per_bio_s(model, pop_offsets) -> float:
@@ -631,10 +636,10 @@ def run_gpu(args):
                         ev_l.append(int(outdeg[spk_np].sum()))
                         nnz_l.append(int(torch.count_nonzero(rring).item()))
                 ms_avg, ev_avg, nnz = float(np.median(ms_l)), float(np.mean(ev_l)), float(np.mean(nnz_l))
-                # own bytes: 9 B per record (target, weight, delay); per sender its list
+                # own bytes: 8 B per (weight, target | delay) record; per sender its list
                 # entry and its two segment offsets in every block's table; 8 B (read +
                 # write) per ring entry updated
-                nbytes = 9 * ev_avg + (4 + 8 * nblk) * nsp + 8 * nnz
+                nbytes = 8 * ev_avg + (4 + 8 * nblk) * nsp + 8 * nnz
                 plain_ms = [p_["ms"] for p_ in sat if p_["spikers"] == nsp]
                 regions.append({"spikers": nsp, "order": order, "events": ev_avg, "ms": ms_avg,
                                 "events_per_s": ev_avg / (ms_avg * 1e-3), "bytes": nbytes,
@@ -762,10 +767,11 @@ def run_gpu(args):
         "roofline": roofline, "kernels": kernels,
         "compressed_records": forms,
         "workloads": extra,
-        "delivery_saturating": {"kernel": "k_deliver_list", "bound": "hbm", "peak": peak, "unit": "GB/s",
-                                "traffic_20480": _recorded_traffic("k_deliver_list"),
+        "delivery_saturating": {"kernel": "k_deliver_slices", "bound": "hbm", "peak": peak, "unit": "GB/s",
+                                "traffic_20480": _recorded_traffic("k_deliver_slices"),
                                 "note": "phase 2 alone over random senders of the same network "
-                                        "(13 B per event + 20 B per sender); int32 red.add into the ring",
+                                        "(13 B per event + 20 B per sender); long lists slice by slice of delays, "
+                                        "summed in shared memory, shorter ones row by row (k_deliver_list)",
                                 "points": sat,
                                 "blocked6": {"kernel": "k_deliver_blocked",
                                              "traffic_20480": _recorded_traffic("k_deliver_blocked"),
@@ -783,7 +789,7 @@ def run_gpu(args):
                                                      "one contiguous read per segment",
                                              "points": forms.get("blocked8", {}).get("delivery_saturating")},
                                 "block_major": {"kernel": "k_deliver_regions",
-                                                "note": "the resident engine's block-major records (9 B per event): "
+                                                "note": "the resident engine's block-major records (8 B per event): "
                                                         "one CTA per target block reads its region's segments; frac "
                                                         "on its own bytes (records, per-sender offsets in every "
                                                         "block's table, 8 B per ring entry updated); random and "
@@ -841,7 +847,7 @@ def main():
     ap.add_argument("--regions", type=int, default=1, help="saturating delivery on block-major records (0: skip)")
     ap.add_argument("--seeds", type=int, default=10, help="network instances timed for the mean RTF (0: none)")
     ap.add_argument("--seed-steps", type=int, default=10, help="bench steps timed per instance")
-    ap.add_argument("--engine", default="resident", choices=["default", "graph", "persistent", "pipelined", "resident"],
+    ap.add_argument("--engine", default="pipelined", choices=["default", "graph", "persistent", "pipelined", "resident"],
                     help="engine of the headline step loop (the resident engine: one launch per 1,024 steps)")
     args = ap.parse_args()
     if args.warmup < 3:
