@@ -753,8 +753,13 @@ struct RegionSource {
     int32_t base;
     int stride;
 
-    // (senders outside the network deliver nothing)
-    __device__ __forceinline__ int32_t sender(int64_t j) const { return __ldcg(list + j) & 0x7FFFFFFF; }
+    // (senders outside the network deliver nothing; the stream takes entries >= 0, so a
+    // negative one becomes one that raw() finds outside)
+    __device__ __forceinline__ int32_t sender(int64_t j) const
+    {
+        const int32_t s = __ldcg(list + j);
+        return s < 0 ? INT32_MAX : s;
+    }
     __device__ __forceinline__ Raw raw(int64_t, int32_t s) const
     {
         if (s >= a.n) return Raw{0, 0};
