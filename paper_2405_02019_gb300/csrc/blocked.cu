@@ -209,7 +209,7 @@ struct BlockedSource {
 // the window marks its first quad, and a lane's block is the last one at or before it.
 // `offs`: the block boundaries, in shared memory; `scratch`: the warp's 32 words.
 template <int FMT>
-__device__ __forceinline__ void blocked_row_window(const StepArgs &a, int64_t t, uint32_t row_quad, uint32_t len,
+__device__ __forceinline__ void blocked_row_window(const StepArgs &a, int64_t t, int64_t row_quad, uint32_t len,
                                                    int32_t s, uint32_t w0, const int32_t *offs, int32_t *scratch)
 {
     constexpr int kPer = 5;  // the table of up to 160 blocks in one round trip
@@ -217,7 +217,7 @@ __device__ __forceinline__ void blocked_row_window(const StepArgs &a, int64_t t,
     const bool ok = w0 + lane < len;
     uint4 va = make_uint4(0, 0, 0, 0), vb = va;
     if (ok) {
-        const uint64_t q = static_cast<uint64_t>(row_quad) + w0 + lane;
+        const int64_t q = row_quad + w0 + lane;
         const uint4 *q16 = reinterpret_cast<const uint4 *>(a.blk_rec);
         if (FMT == SNN_RECORD_BLOCKED8) {
             va = __ldcs(q16 + 2 * q);
@@ -313,17 +313,18 @@ __global__ void __launch_bounds__(kThreads, 1024 / kThreads)
         for (int64_t it = gw; it < nspk * a.row_windows; it += warps) {
             const int64_t j = it / a.row_windows;
             const uint32_t w0 = static_cast<uint32_t>(it - j * a.row_windows) * 32;
-            uint32_t row_quad, len;
+            int64_t row_quad;
+            uint32_t len;
             int32_t s;
             if (list != nullptr) {
                 s = __ldcg(spk + j);
                 const int64_t rs = __ldg(a.row_ptr + s);
-                row_quad = static_cast<uint32_t>(rs / kBlockQuad);
+                row_quad = rs / kBlockQuad;
                 len = static_cast<uint32_t>((__ldg(a.row_ptr + s + 1) - rs) / kBlockQuad);
             } else {
                 const int4 e = it == gw ? first : __ldcg(reinterpret_cast<const int4 *>(a.queue + (t & 1) * a.npad + j));
-                row_quad = static_cast<uint32_t>(e.x);
-                len = static_cast<uint32_t>(e.y);
+                row_quad = entry_first_quad(e.x, e.y);
+                len = entry_quads(e.y);
                 s = e.z;
             }
             if (w0 < len)

@@ -7,6 +7,7 @@
 #include <vector>
 
 #include "../../include/snn.h"
+#include "philox.cuh"
 
 namespace snn {
 
@@ -38,14 +39,31 @@ struct alignas(64) Ctl {
     uint32_t pad[5];
 };
 
-// Pipelined engine: one queue entry per spike of a step, written by the thread that
-// decided the spike, consumed by the next kernel's delivery warps.
+// Pipelined and graph engines: one queue entry per spike of a step, written by the thread that
+// decided the spike, consumed by the delivery warps.  Rows are whole quads of four records; a
+// row has fewer than 2^31 records (row lengths are int32), so its length in quads leaves
+// three bits for the first quad's upper bits: 35 in all, 2^37 records, above what a network
+// may have (2^35 synapses in a batch, and up to three records of padding per row).
+constexpr int kEntryLenBits = 29;
 struct alignas(16) QueueEntry {
-    uint32_t row_quad;   // first synapse of the row / 4
-    uint32_t len_quads;  // padded row length / 4
+    uint32_t row_quad;   // low 32 bits of the row's first quad
+    uint32_t len_quads;  // its quads; above, bits 32 to 34 of the first one
     int32_t neuron;
     int32_t step;        // low 32 bits of the step index (tells fresh entries from stale ones)
 };
+SNN_HD QueueEntry queue_entry(int64_t row_begin, int64_t row_end, int32_t neuron, int64_t step)
+{
+    const uint64_t q = static_cast<uint64_t>(row_begin) >> 2;
+    return QueueEntry{static_cast<uint32_t>(q),
+                      static_cast<uint32_t>((row_end - row_begin) >> 2) | (static_cast<uint32_t>(q >> 32) << kEntryLenBits),
+                      neuron, static_cast<int32_t>(step)};
+}
+// From an entry's first two words
+SNN_HD int64_t entry_first_quad(uint32_t row_quad, uint32_t len_quads)
+{
+    return static_cast<int64_t>((static_cast<uint64_t>(len_quads >> kEntryLenBits) << 32) | row_quad);
+}
+SNN_HD uint32_t entry_quads(uint32_t len_quads) { return len_quads & ((1u << kEntryLenBits) - 1u); }
 
 // int8 read-back of one (source, target) population pair: w = base + code * step.
 struct alignas(8) PairQ {

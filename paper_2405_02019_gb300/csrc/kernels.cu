@@ -245,11 +245,7 @@ __device__ __forceinline__ void append_spikes(const StepArgs &a, int64_t t, int6
                 atomicOr(&a.ctl->err, kErrRaster);
             }
             if (pos - begin < static_cast<uint32_t>(a.queue_cap)) {
-                QueueEntry e;
-                e.row_quad = static_cast<uint32_t>(rp[j] >> 2);
-                e.len_quads = static_cast<uint32_t>((rp[j + 1] - rp[j]) >> 2);
-                e.neuron = static_cast<int32_t>(i0 + j);
-                e.step = static_cast<int32_t>(t);
+                const QueueEntry e = queue_entry(rp[j], rp[j + 1], static_cast<int32_t>(i0 + j), t);
                 *reinterpret_cast<int4 *>(a.queue + (t & 1) * a.npad + (pos - begin)) = *reinterpret_cast<const int4 *>(&e);
             }
             ++pos;
@@ -393,8 +389,8 @@ __device__ __forceinline__ void deliver_rows_fmt(const StepArgs &a, int64_t t, i
     for (int64_t it = warp; it < nspk * ipj; it += nwarps) {
         const int64_t j = it / ipj, part = it - j * ipj;
         const int4 raw = it == warp && ipj == cpr ? first : __ldcg(reinterpret_cast<const int4 *>(rows + j));
-        const int64_t rs = static_cast<int64_t>(static_cast<uint32_t>(raw.x)) * 4;
-        const int64_t re = rs + static_cast<int64_t>(static_cast<uint32_t>(raw.y)) * 4;
+        const int64_t rs = entry_first_quad(raw.x, raw.y) * 4;
+        const int64_t re = rs + static_cast<int64_t>(entry_quads(raw.y)) * 4;
         const int src = FMT == SNN_RECORD_PACKED_I8 ? __ldg(a.pop_id + raw.z) : 0;
         for (int64_t c = part * per, off = rs + c * kChunk; c < (part + 1) * per && off < re; ++c, off += kChunk)
             deliver_chunk<FMT>(a, t, off, re, src);
@@ -615,11 +611,7 @@ __device__ __forceinline__ void pipe_quad(const StepArgs &a, const int64_t &t, i
         if (!spk[j]) continue;
         const int64_t rs = rp[j];
         const int64_t re = rp[j + 1];
-        QueueEntry e;
-        e.row_quad = static_cast<uint32_t>(rs >> 2);
-        e.len_quads = static_cast<uint32_t>((re - rs) >> 2);
-        e.neuron = static_cast<int32_t>(i0 + j);
-        e.step = static_cast<int32_t>(sn);
+        const QueueEntry e = queue_entry(rs, re, static_cast<int32_t>(i0 + j), sn);
         *reinterpret_cast<int4 *>(region + k) = *reinterpret_cast<const int4 *>(&e);
         ++k;
         prefetch_row(a, rs, re);
@@ -697,8 +689,8 @@ __device__ __forceinline__ void pipe_deliver_fmt(const StepArgs &a, const int64_
                 a.rast_t[pos] = static_cast<int32_t>(t);
             }
         }
-        const int64_t rs = static_cast<int64_t>(static_cast<uint32_t>(raw.x)) * 4;
-        const int64_t re = rs + static_cast<int64_t>(static_cast<uint32_t>(raw.y)) * 4;
+        const int64_t rs = entry_first_quad(raw.x, raw.y) * 4;
+        const int64_t re = rs + static_cast<int64_t>(entry_quads(raw.y)) * 4;
         const int src = FMT == SNN_RECORD_PACKED_I8 ? sender_pop(a, raw.z) : 0;
         for (int64_t c = part * per, off = rs + c * kChunk; c < (part + 1) * per && off < re; ++c, off += kChunk)
             deliver_chunk<FMT>(a, ph, off, re, src);

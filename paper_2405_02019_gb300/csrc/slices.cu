@@ -32,6 +32,9 @@ namespace snn {
 namespace {
 
 constexpr int kSliceThreads = 768;
+// (the stream counts units in 32 bits: a plan has at most kSliceMaxParts kSliceCells rows of at
+// most 65,535 synapses, padded to quads)
+static_assert(int64_t{kSliceMaxParts} * kSliceCells * 65536 / 4 < int64_t{1} << 32, "units of a sliced network");
 constexpr int kSliceWarps = kSliceThreads / 32;
 constexpr int kSliceRounds = 2;
 constexpr size_t kSliceSmem = sizeof(int32_t) * kSliceCells + sizeof(uint2) * 32 * kSliceRounds * kSliceWarps;
