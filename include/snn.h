@@ -254,7 +254,7 @@ typedef struct snn_info {
     int64_t n_neurons;
     int64_t n_synapses;
     int64_t n_synapses_padded;
-    int64_t t;            /* steps enqueued so far */
+    int64_t t;            /* steps enqueued so far (once steps were captured: steps that have run) */
     int64_t spikes_read;  /* spikes of completed steps moved to the host so far */
     int64_t events_read;  /* recurrent synaptic events (sum of the senders' out-degrees) of those */
     int32_t n_pops;
@@ -319,8 +319,16 @@ int snn_export_network(const snn_spec *spec, int64_t *row_ptr, int32_t *post, in
 
 /* Enqueues n_steps steps (Listing push / push2 of §3.1; one step = dt) on
  * `cuda_stream` and returns without waiting.  n_steps = 0 is a no-op.
+ * On a stream that the caller is capturing the steps become part of the caller's graph:
+ * nothing runs and no step is counted until it is replayed, and every replay runs n_steps
+ * more steps from wherever the network stands.  The library does not see replays: let them
+ * finish before a call that reads the network (or queue them on the legacy stream, which
+ * those calls wait for), and do not change the schedule or the grouping between capture and
+ * replay.
  * Errors: SNN_EINVAL (n_steps < 0), SNN_ESTATE (after a sticky device error),
- * SNN_ECUDA.  A persistent-engine barrier that waits longer than 2 s records a device
+ * SNN_ENOTSUP (graph and pipelined engines: a captured call of steps_per_graph steps or
+ * more, on the pipelined engine counted from the next multiple of 64 steps; nothing is
+ * enqueued), SNN_ECUDA.  A persistent-engine barrier that waits longer than 2 s records a device
  * error that the next read reports as SNN_ETIMEOUT. */
 int snn_step_n(snn_net *net, int64_t n_steps, void *cuda_stream);
 
@@ -353,7 +361,9 @@ int snn_collect_spikes(snn_net *net, int64_t *steps, int32_t *neurons, int64_t c
 int snn_read_rates(snn_net *net, int64_t t_begin, int64_t t_end, double *pop_rates_hz, int32_t *neuron_counts);
 
 /* Fills `out` with the network's constants (the FP64 and FP32 propagators of §2.2, the
- * thalamic Poisson tables) and counters (host only, no wait).  No passage of its own:
+ * thalamic Poisson tables) and counters (host only, no wait; after a captured snn_step_n
+ * it waits for the enqueued steps and takes their count from the device, as does
+ * snn_get_layout).  No passage of its own:
  * ABI helper.  Errors: SNN_EINVAL (null argument). */
 int snn_get_info(const snn_net *net, snn_info *out);
 

@@ -94,6 +94,9 @@ struct snn_net {
     uint32_t *snap_ctl = nullptr;
     bool snap_fresh = false;       // the latest snapshot is where the device stands when it is done
     bool drained = false;          // nothing was enqueued since the last drain
+    // a caller captured steps of this handle: replays of that graph enqueue steps unseen, so
+    // the step count, the cursor and the error bits are the device's, never these copies
+    bool captured = false;
     cudaEvent_t snap_ev[kSnaps] = {};
     int64_t snap_t[kSnaps] = {};   // steps enqueued at each snapshot
     int64_t n_snaps = 0;           // snapshots recorded
@@ -387,6 +390,41 @@ int wait_done(snn_net *net)
     return SNN_OK;
 }
 
+// The control block after the steps that have finished.  Taken in the relaxed capture mode, so
+// that a capture elsewhere (snn_get_info between captured calls) stays valid; the copy waits
+// for the legacy stream's work like any plain cudaMemcpy, unless a capture forbids using it.
+int read_ctl(const snn_net *net, snn::Ctl &ctl)
+{
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    SNN_CUDA_TRY(cudaThreadExchangeStreamCaptureMode(&mode));
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaSuccess;
+    if (net->n_snaps > 0) e = cudaEventSynchronize(net->snap_ev[(net->n_snaps - 1) % snn_net::kSnaps]);
+    if (e == cudaSuccess) {
+        if (cudaStreamIsCapturing(cudaStreamLegacy, &status) == cudaSuccess) {
+            e = cudaMemcpy(&ctl, net->arena + net->L.ctl, sizeof(ctl), cudaMemcpyDeviceToHost);
+        } else {
+            cudaGetLastError();
+            e = cudaMemcpyAsync(&ctl, net->arena + net->L.ctl, sizeof(ctl), cudaMemcpyDeviceToHost, net->copy_stream);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(net->copy_stream);
+        }
+    }
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (e != cudaSuccess) return fail(SNN_ECUDA, std::string("control block: ") + cudaGetErrorString(e));
+    return SNN_OK;
+}
+
+// Steps enqueued so far; of a captured handle, the steps that have finished.
+int count_steps(const snn_net *net, int64_t &t)
+{
+    t = net->t;
+    if (!net->captured) return SNN_OK;
+    snn::Ctl ctl;
+    const int rc = read_ctl(net, ctl);
+    if (rc == SNN_OK) t = ctl.t_base;
+    return rc;
+}
+
 // Pinned staging for at least `want` entries of each of the raster's two arrays.
 int reserve_pinned(snn_net *net, int64_t want)
 {
@@ -519,7 +557,13 @@ int drain_steps(snn_net *net)
     if (rc) return rc;
     if (!net->drained) {
         uint32_t end[4];  // Ctl: cursor, step_begin[2], err
-        if (net->snap_fresh) {
+        if (net->captured) {
+            snn::Ctl ctl;
+            rc = read_ctl(net, ctl);
+            if (rc) return rc;
+            std::memcpy(end, &ctl.cursor, sizeof(end));
+            net->t = ctl.t_base;
+        } else if (net->snap_fresh) {
             std::memcpy(end, net->snap_ctl + 4 * ((net->n_snaps - 1) % snn_net::kSnaps), sizeof(end));
         } else {
             SNN_CUDA_TRY(cudaMemcpy(end, net->arena + net->L.ctl + offsetof(snn::Ctl, cursor), sizeof(end),
@@ -537,7 +581,7 @@ int drain_steps(snn_net *net)
         }
         net->raster_read = 0;
         net->snaps_valid_from = net->n_snaps;  // their cursors refer to the raster before the reset
-        net->drained = true;
+        net->drained = !net->captured;
     }
     if (net->device_error & snn::kErrTimeout)
         return fail(SNN_ETIMEOUT, "a bounded device wait (persistent barrier or resident mailbox) timed out");
@@ -561,6 +605,7 @@ int drain(snn_net *net)
 // two more calls' spikes are written before the next chance.
 int collect(snn_net *net)
 {
+    if (net->captured) return drain(net);
     const int64_t j = net->n_snaps - 2;
     if (j < 0 || j < net->snaps_valid_from) return SNN_OK;
     const int slot = static_cast<int>(j % snn_net::kSnaps);
@@ -1005,19 +1050,30 @@ int snn_step_n(snn_net *net, int64_t n_steps, void *cuda_stream)
     if (net->device_error) return fail(SNN_ESTATE, "a previous device error is pending");
     if (n_steps == 0) return SNN_OK;
     cudaStream_t st = static_cast<cudaStream_t>(cuda_stream);
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(st, &status) != cudaSuccess) cudaGetLastError();
+    const bool capturing = status != cudaStreamCaptureStatusNone;
+    const bool one_launch = net->engine == SNN_ENGINE_PERSISTENT || net->engine == SNN_ENGINE_RESIDENT;
+    if (capturing && !one_launch) {
+        // a graph launch cannot be captured, so a caller that captures this stream gets the
+        // steps as launches; a run of a step graph's length and more (from the next multiple
+        // of the phase period on) is refused before anything is enqueued
+        const int64_t head = net->engine == SNN_ENGINE_PIPELINED
+                                 ? (snn::kPhasePeriod - net->t % snn::kPhasePeriod) % snn::kPhasePeriod
+                                 : 0;
+        if (n_steps - head >= net->steps_per_graph)
+            return fail(SNN_ENOTSUP, "a captured call must be shorter than steps_per_graph");
+    }
+    if (capturing) net->captured = true;
     net->drained = false;
     net->snap_fresh = false;
-    if (net->engine == SNN_ENGINE_PERSISTENT || net->engine == SNN_ENGINE_RESIDENT) {
+    if (one_launch) {
         const int rc = net->engine == SNN_ENGINE_RESIDENT ? launch_steps_resident(net, n_steps, st)
                                                           : launch_steps_persistent(net, n_steps, st);
         if (rc) return rc;
     } else {
         int64_t n = n_steps;
-        // a caller that captures this stream gets the steps as launches (a graph launch cannot
-        // be captured)
-        cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
-        if (cudaStreamIsCapturing(st, &capture) != cudaSuccess) cudaGetLastError();
-        if (capture == cudaStreamCaptureStatusNone)
+        if (!capturing)
             for (const auto &g : net->graphs)
                 for (; n >= g.steps; n -= g.steps) SNN_CUDA_TRY(cudaGraphLaunch(g.exec, st));
         if (n > 0) {
@@ -1025,6 +1081,7 @@ int snn_step_n(snn_net *net, int64_t n_steps, void *cuda_stream)
             if (rc) return rc;
         }
     }
+    if (capturing) return SNN_OK;  // nothing has run; a replay's steps are counted on the device
     net->t += n_steps;
     // where the raster and the error bits stand after these steps
     const int slot = static_cast<int>(net->n_snaps % snn_net::kSnaps);
@@ -1172,8 +1229,11 @@ int snn_read_rates(snn_net *net, int64_t t_begin, int64_t t_end, double *pop_rat
     HandleScope scope(net);
     if (!net || !pop_rates_hz) return fail(SNN_EINVAL, "null argument");
     if (t_begin < 0 || t_end <= t_begin) return fail(SNN_EINVAL, "empty or negative window");
-    if (t_end > net->t) return fail(SNN_EINVAL, "window ends after the steps enqueued so far");
-    int rc = drain(net);
+    int64_t t_now = 0;
+    int rc = count_steps(net, t_now);
+    if (rc) return rc;
+    if (t_end > t_now) return fail(SNN_EINVAL, "window ends after the steps enqueued so far");
+    rc = drain(net);
     const int P = net->spec.model.n_pops;
     std::vector<int64_t> pop_cnt(P, 0);
     if (neuron_counts) std::fill(neuron_counts, neuron_counts + net->n, 0);
@@ -1198,14 +1258,17 @@ int snn_get_info(const snn_net *net, snn_info *out)
 {
     if (!net || !out) return fail(SNN_EINVAL, "null argument");
     std::memset(out, 0, sizeof(*out));
+    int64_t t_now = 0;
+    const int rc = count_steps(net, t_now);
+    if (rc) return rc;
     out->n_neurons = net->n;
     out->n_synapses = net->n_syn;
     out->n_synapses_padded = net->n_syn_padded;
-    out->t = net->t;
+    out->t = t_now;
     // count spikes of completed steps only (the pipelined engine records the next
     // step's spikes one launch early)
     const int64_t done_end =
-        std::lower_bound(net->hist_t.begin(), net->hist_t.end(), static_cast<int32_t>(std::min<int64_t>(net->t, INT32_MAX))) -
+        std::lower_bound(net->hist_t.begin(), net->hist_t.end(), static_cast<int32_t>(std::min<int64_t>(t_now, INT32_MAX))) -
         net->hist_t.begin();
     int64_t pending_events = 0;
     for (size_t j = static_cast<size_t>(done_end); j < net->hist_t.size(); ++j) pending_events += net->out_degree[net->hist_i[j]];
@@ -1251,10 +1314,13 @@ int snn_get_layout(const snn_net *net, snn_layout *out)
 {
     if (!net || !out) return fail(SNN_EINVAL, "null argument");
     const snn::Layout &L = net->L;
+    int64_t t_now = 0;
+    const int rc = count_steps(net, t_now);
+    if (rc) return rc;
     out->ctl = L.ctl;
     out->params = L.tables;
     const bool second = (net->engine == SNN_ENGINE_PIPELINED || net->engine == SNN_ENGINE_PERSISTENT) &&
-                        ((net->t - 1) & 1);
+                        ((t_now - 1) & 1);
     out->U = second ? L.U2 : L.U;
     out->I = L.I;
     out->R = second ? L.R2 : L.R;
@@ -1425,6 +1491,8 @@ int snn_set_circuit_groups(snn_net *net, int32_t circuits_per_group)
         return fail(SNN_ENOTSUP, "circuit groups run on the graph and pipelined engines");
     if (net->device_error) return fail(SNN_ESTATE, "a previous device error is pending");
     int rc = wait_done(net);
+    if (rc) return rc;
+    rc = count_steps(net, net->t);  // the pending spikes' queue is t mod 4
     if (rc) return rc;
     const int32_t old = net->circuits_per_group;
     net->circuits_per_group = circuits_per_group >= static_cast<int32_t>(net->circuits.size()) ? 0 : circuits_per_group;
