@@ -285,6 +285,15 @@ bool validate_spec(const snn_spec &spec, std::string &why)
     return true;
 }
 
+// Whether the network keeps the table of where each delay starts in every row (128 bytes a
+// neuron): only lists on rows that can be delivered by slices read it (make_slice_plan).
+static bool wants_delay_table(const snn_spec &spec)
+{
+    const int64_t npad = (count_neurons(spec) + kNeuronAlign - 1) / kNeuronAlign * kNeuronAlign;
+    return !is_blocked(spec.record_format) && spec.engine != SNN_ENGINE_RESIDENT &&
+           npad <= int64_t{kSliceMaxParts} * kSliceCells;
+}
+
 Layout make_layout(const snn_spec &spec)
 {
     auto up = [](uint64_t x) { return (x + 255) & ~uint64_t{255}; };
@@ -347,8 +356,7 @@ Layout make_layout(const snn_spec &spec)
     L.sort_cur = o; o = up(o + 4 * (kRasterSortMaxSteps + 1));
     L.sort_off = o; o = up(o + 4 * (kRasterSortMaxSteps + 2));
     L.sort_out = o; o = up(o + 4 * std::min(L.rast_cap, kRasterSortMax));
-    // where each delay starts in every row (the layouts that keep rows in delay order)
-    L.row_delay = o; o = up(o + (is_blocked(fmt) || resident ? 0 : 2 * uint64_t{kDMax} * n));
+    L.row_delay = o; o = up(o + (wants_delay_table(spec) ? 2 * uint64_t{kDMax} * n : 0));
     L.total = o;
     return L;
 }
@@ -748,13 +756,13 @@ bool block_major_records(HostNetwork &net, int64_t width, int nthreads, std::str
     return true;
 }
 
-bool build_one(const snn_spec &spec, const Constants &c, HostNetwork &net, std::string &why, int num_sms);
+bool build_one(const snn_spec &spec, const Constants &c, HostNetwork &net, std::string &why, int num_sms, bool delay_table);
 }
 
 bool build_host_network(const snn_spec &spec, const Constants &c, HostNetwork &net, std::string &why, int num_sms)
 {
     if (spec.n_circuits <= 0) {
-        if (!build_one(spec, c, net, why, num_sms)) return false;
+        if (!build_one(spec, c, net, why, num_sms, wants_delay_table(spec))) return false;
         net.circuits = {CircuitInfo{0, net.n, spec.seed, 0}};
         if (spec.engine == SNN_ENGINE_RESIDENT && num_sms > 0) {
             const int64_t width = resident_width(net.n, num_sms);
@@ -782,12 +790,12 @@ bool build_host_network(const snn_spec &spec, const Constants &c, HostNetwork &n
         all.d.reserve(s_all);
     }
     int64_t base = 0;
-    bool delay_table = true;
+    bool delay_table = wants_delay_table(spec);
     for (int ci = 0; ci < spec.n_circuits; ++ci) {
         snn_spec one = circuit_spec(spec, ci);
         one.record_format = SNN_RECORD_PLAIN9;
         HostNetwork h;
-        if (!build_one(one, c, h, why, 0)) return false;
+        if (!build_one(one, c, h, why, 0, delay_table)) return false;
         if (ci > 0) base = (all.n + 127) / 128 * 128;
         // neurons: gap (inert) then the circuit
         const int64_t syn_base = all.row_ptr.empty() ? 0 : all.row_ptr.back();
@@ -833,7 +841,7 @@ bool build_host_network(const snn_spec &spec, const Constants &c, HostNetwork &n
 
 namespace {
 
-bool build_one(const snn_spec &spec, const Constants &c, HostNetwork &net, std::string &why, int num_sms)
+bool build_one(const snn_spec &spec, const Constants &c, HostNetwork &net, std::string &why, int num_sms, bool delay_table)
 {
     const int nthreads = resolve_threads(spec.n_threads);
     const snn_model &m = spec.model;
@@ -939,9 +947,9 @@ bool build_one(const snn_spec &spec, const Constants &c, HostNetwork &net, std::
     net.tgt.assign(net.n_syn_padded, 0);
     net.w.assign(net.n_syn_padded, 0);
     net.d.assign(net.n_syn_padded, 1);
-    // where each delay starts in its row, and the synapses of each delay, for the layouts
-    // that keep the delay order (16-bit offsets: no longer rows)
-    const bool delay_table = !is_blocked(spec.record_format) && spec.engine != SNN_ENGINE_RESIDENT && maxrow <= 65535;
+    // where each delay starts in its row, and the synapses of each delay (16-bit offsets: no
+    // longer rows)
+    delay_table = delay_table && maxrow <= 65535;
     if (delay_table) net.row_delay.resize(static_cast<size_t>(n) * kDMax);
     std::vector<std::array<int64_t, kDMax>> delay_events(std::max(1, nthreads), std::array<int64_t, kDMax>{});
     parallel_for(nthreads, n, [&](int th, int64_t lo, int64_t hi) {

@@ -292,7 +292,7 @@ struct HostNetwork {
     std::vector<int32_t> w;
     std::vector<uint8_t> d;
     std::vector<float> u0;
-    std::vector<uint16_t> row_delay;  // rows in delay order: [n][64] where each delay starts, entry 0 the row's end (empty if a row is too long)
+    std::vector<uint16_t> row_delay;  // rows in delay order: [n][64] where each delay starts, entry 0 the row's end (empty if no list needs it or a row is too long)
     int64_t delay_events[kDMax] = {}; // synapses of each delay
     std::vector<int32_t> blk;      // blocked records: block boundaries
     std::vector<uint16_t> rec16;   // blocked records: local target | delay << 10
