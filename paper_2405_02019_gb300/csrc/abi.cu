@@ -349,7 +349,10 @@ int capture_steps(snn_net *net, int64_t steps, cudaGraphExec_t *exec)
     if (rc == SNN_OK) {
         cudaError_t e = cudaGraphInstantiate(exec, g, 0);
         // to the device now: the first replay would otherwise pay for it (60 us in a call of 10 steps)
-        if (e == cudaSuccess) e = cudaGraphUpload(*exec, net->capture_stream);
+        if (e == cudaSuccess) {
+            e = cudaGraphUpload(*exec, net->capture_stream);
+            if (e != cudaSuccess) cudaGraphExecDestroy(*exec);  // the caller keeps it only on success
+        }
         if (e != cudaSuccess) rc = fail(SNN_ECUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
     }
     if (g) cudaGraphDestroy(g);
