@@ -4,7 +4,8 @@ One bench step = 1,024 simulation steps of 0.1 ms (102.4 ms of biological time: 
 CUDA-graph replay of the pipelined engine, by default, or one launch of the resident engine)
 of the full microcircuit (77,169 neurons, 284,811,022 synapses,
 seed 1 + rank), so the default --steps 100 covers the paper's 10 s runs (§4).  Prints
-one JSON line.
+one JSON line of about 2,300 characters, the headline; the whole record, of about 20,000,
+goes to standard error.
 
   value     recurrent synaptic events/s (sum of the spikers' out-degrees / seconds),
             device-timed with CUDA events around the snn_step_n calls
@@ -19,7 +20,8 @@ one JSON line.
   cpu_baseline  the CPU oracle (single thread) on a bounded sample of the workload,
             and in its `multithreaded` entry the same step on every host core
   energy    the GPU board's energy counter over the timed region / recurrent events
-Further objects: delivery_saturating (phase 2 alone over 2,048-20,480 random senders,
+Further objects, one or two numbers of each in the headline (longest_lists, forms_rtf,
+workloads_us_per_step): delivery_saturating (phase 2 alone over 2,048-20,480 random senders,
 plain and target-blocked records), compressed_records (int8, bf16, blocked forms) and
 workloads (32 uneven circuits in autotuned circuit groups; the 4x-scale circuit in
 plain and int8 records).
@@ -90,6 +92,49 @@ def _recorded_traffic(kernel: str):
     if rec is None or src is None or rec.get("sources_sha256_16") != _kernel_sources_hash(src):
         return None
     return rec.get("dram_bytes_per_launch")
+
+
+def _digits(x, n=8):
+    """Floats of a record to n significant digits."""
+    if isinstance(x, dict):
+        return {k: _digits(v, n) for k, v in x.items()}
+    if isinstance(x, (list, tuple)):
+        return [_digits(v, n) for v in x]
+    return float(f"{x:.{n}g}") if isinstance(x, float) else x
+
+
+def headline(rec: dict) -> dict:
+    """The part of a run's record that fits one short line of output: every key of the
+    measured workload, and one number or two of each other section."""
+    def pick(d, *keys):
+        return {k: d[k] for k in keys if k in d}
+
+    def longest(points):  # of the saturating lists
+        if not points:
+            return None
+        top = max(p["spikers"] for p in points)
+        return {p.get("order", "random"): pick(p, "ms", "frac") for p in points if p["spikers"] == top}
+
+    out = {k: v for k, v in rec.items() if not isinstance(v, (dict, list))}
+    out["config"] = rec["config"]
+    out["e2e"] = {k: v for k, v in rec["e2e"].items() if k != "note"}
+    out["clocks"] = rec["clocks"]
+    out["roofline"] = rec["roofline"]
+    out["kernels"] = {k: pick(v, "avg_us", "us_per_step") for k, v in rec["kernels"].items()}
+    if rec.get("cpu_baseline"):
+        out["cpu_baseline"] = pick(rec["cpu_baseline"], "value", "unit", "cores", "kind", "rtf")
+        mt = rec["cpu_baseline"].get("multithreaded") or {}
+        out["cpu_baseline"]["multithreaded"] = pick(mt, "value", "cores", "rtf")
+    if rec.get("energy"):
+        out["energy"] = pick(rec["energy"], "joules", "nj_per_event")
+    if rec.get("instances"):
+        out["instances"] = pick(rec["instances"], "n", "rtf_mean", "rtf_sd")
+    out["forms_rtf"] = {k: v["rtf"] for k, v in rec["compressed_records"].items()}
+    out["workloads_us_per_step"] = {k: v["us_per_step"] for k, v in rec["workloads"].items()}
+    sat = rec["delivery_saturating"]
+    lists = {"rows": sat["points"], **{k: v["points"] for k, v in sat.items() if isinstance(v, dict)}}
+    out["longest_lists"] = {k: longest(v) for k, v in lists.items() if v}
+    return _digits(out)
 
 
 def thalamic_events_per_bio_s(model, pop_offsets) -> float:
@@ -816,7 +861,8 @@ def run_gpu(args):
     if cpu is not None:
         line["cpu_baseline"] = cpu
     if rank == 0:
-        print(json.dumps(line), flush=True)
+        print(json.dumps(line), file=sys.stderr, flush=True)
+        print(json.dumps(headline(line)), flush=True)
     return 0
 
 
