@@ -56,28 +56,42 @@ WORKLOAD = "pd_full"
 METRIC = "synaptic events/s and real-time factor (full microcircuit, 1 GB300), % HBM roofline"
 
 
+CSRC = os.path.join(ROOT, "paper_2405_02019_gb300", "csrc")
+
+
 def _kernel_sources_hash(files=("kernels.cu", "internal.hpp")) -> str:
     """Hash of the code lines (comment-only and blank lines ignored) of kernel sources."""
     import hashlib
 
-    csrc = os.path.join(ROOT, "paper_2405_02019_gb300", "csrc")
     lines = []
     for f in files:
-        for line in open(os.path.join(csrc, f), encoding="utf-8"):
+        for line in open(os.path.join(CSRC, f), encoding="utf-8"):
             code = line.strip()
             if code and not code.startswith("//"):
                 lines.append(code)
     return hashlib.sha256("\n".join(lines).encode()).hexdigest()[:16]
 
 
-# the sources each recorded kernel is built from
-_SOURCES = {
-    "k_step": ("kernels.cu", "launch.cuh", "internal.hpp"),
-    "k_deliver_slices": ("slices.cu", "stream.cuh", "internal.hpp"),
-    "k_deliver_blocked": ("blocked.cu", "stream.cuh", "internal.hpp"),
-    "k_resident": ("resident.cu", "stream.cuh", "internal.hpp"),
-    "k_deliver_regions": ("resident.cu", "stream.cuh", "internal.hpp"),
-}
+# the file each recorded kernel stands in
+_SOURCES = {"k_step": "kernels.cu", "k_deliver_slices": "slices.cu", "k_deliver_blocked": "blocked.cu",
+            "k_resident": "resident.cu", "k_deliver_regions": "resident.cu"}
+
+
+def _kernel_sources(kernel: str):
+    """The files a recorded kernel is built from: its own and every header beside it that it
+    includes, directly or through another; None for a kernel that is not recorded."""
+    import re
+
+    own = next((f for k, f in _SOURCES.items() if kernel.startswith(k)), None)
+    if own is None:
+        return None
+    todo, headers = [own], set()
+    while todo:
+        text = open(os.path.join(CSRC, todo.pop()), encoding="utf-8").read()
+        new = {h for h in re.findall(r'^#include "([^"/]+)"', text, re.M)} - headers
+        headers |= new
+        todo += new
+    return (own, *sorted(headers))
 
 
 def _recorded_traffic(kernel: str):
@@ -88,7 +102,7 @@ def _recorded_traffic(kernel: str):
     if not os.path.exists(p):
         return None
     rec = json.load(open(p)).get(kernel)
-    src = next((f for k, f in _SOURCES.items() if kernel.startswith(k)), None)
+    src = _kernel_sources(kernel)
     if rec is None or src is None or rec.get("sources_sha256_16") != _kernel_sources_hash(src):
         return None
     return rec.get("dram_bytes_per_launch")
