@@ -384,6 +384,9 @@ int capture_graph(snn_net *net)
         if (rc) return rc;
         net->graphs.push_back({m, exec});
     }
+    // CUDA orders an upload behind earlier launches of its graph, and promises nothing for
+    // launches in other streams that follow
+    SNN_CUDA_TRY(cudaStreamSynchronize(net->capture_stream));
     return SNN_OK;
 }
 
