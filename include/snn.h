@@ -112,7 +112,8 @@ typedef struct snn_circuit {
  *     scale_n / 1000); pair counts K_ab = round(p[b][a] * (N_full_a * scale_k / 1000) * N_b),
  *     the paper's expected count N_pre N_post p (§2.2);
  *   seed: network, initial-state and thalamic streams (Philox4x64-10);
- *   steps_per_graph: steps captured in one CUDA graph (0 = 1000);
+ *   steps_per_graph: steps captured in the longest CUDA graph (0 = 1000; pipelined engine:
+ *     0 = 1024, and a multiple of 64, rounded down, at least 64);
  *   raster_capacity: spikes the device holds between reads (0 = 1<<24);
  *   deliver_blocks: CTAs of the delivery kernel (0 = 2 per SM);
  *   custom: NULL, or an explicit network (then the scales are ignored);
@@ -295,8 +296,8 @@ int snn_query_sizes(const snn_spec *spec, snn_sizes *out);
  * every population pair drawn with replacement, §2.2; rows grouped by sender and
  * sorted by delay, the indexed store of §3.5), uploads it into the caller's device
  * arena on `cuda_stream`, initialises U from the u_init Gaussians, I = R = 0, the
- * ring to zero, and captures the step loop into a CUDA graph (graph and pipelined
- * engines; the persistent engine launches its steps directly).  Returns when the
+ * ring to zero, and captures the step loop into CUDA graphs of four lengths (graph and
+ * pipelined engines; the persistent engine launches its steps directly).  Returns when the
  * upload is complete.  On success *out owns host-side state; free it with
  * snn_destroy.  Errors: SNN_EINVAL (spec), SNN_ENOMEM (host memory, or arena_bytes
  * below snn_query_sizes' figure), SNN_ECUDA. */
@@ -433,11 +434,13 @@ int snn_load_state(snn_net *net, const void *host_buf, uint64_t bytes);
 /* Phase 2 of Listing push2 (§3.1) alone, for measurement and tests: adds every
  * synapse of the senders spikers[0 .. n_spikers) (device int32 neuron ids, each
  * below n_neurons; repeats allowed) into the ring as spikes of step t, i.e.
- * W[(t + d) mod 64][target] += w, in one launch of `blocks` CTAs (0 = full
- * occupancy; the blocked formats and the resident engine's block-major records always
- * launch one CTA per target block, which reads only its block's segments) on
- * `cuda_stream`; returns without waiting.  The ring keeps the added
- * input, so the simulated dynamics change accordingly.
+ * W[(t + d) mod 64][target] += w, in one launch of `blocks` CTAs on `cuda_stream`;
+ * returns without waiting.  blocks = 0 chooses the launch: on rows, full occupancy for
+ * short lists, and one CTA per SM that sums a slice of delays for long ones; the blocked
+ * formats and the resident engine's block-major records always launch one CTA per target
+ * block, which reads only its block's segments.  (Block-major records: ids outside the
+ * network deliver nothing.)  The ring keeps the added input, so the simulated dynamics
+ * change accordingly.
  * Errors: SNN_EINVAL (null or negative arguments), SNN_ECUDA. */
 int snn_deliver_spikes(snn_net *net, const int32_t *spikers, int64_t n_spikers, int64_t t, int32_t blocks,
                        void *cuda_stream);

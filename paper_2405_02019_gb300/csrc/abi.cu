@@ -1,9 +1,10 @@
 // C ABI of the simulator: network setup, the CUDA-graph step engine and raster readout.
 //
-// The step engine captures `steps_per_graph` steps (each: k_update then k_deliver,
-// the two phases of Listing push2, §3.1) plus one counter advance into a CUDA graph
-// at build time and replays it; remainders are launched directly.  The step index
-// lives on the device (Ctl::t_base), so a replay needs no host-side parameter update
+// The graph and pipelined engines capture steps (Listing push2, §3.1: k_update and the
+// delivery kernel, or one k_step) plus one counter advance into CUDA graphs at build time: one
+// of `steps_per_graph` steps and shorter ones of 128, 32 and 8.  A run replays the longest that
+// fits again and again; fewer than the shortest one's steps are launched one by one.  The step
+// index lives on the device (Ctl::t_base), so a replay needs no host-side parameter update
 // and no host round trip happens between steps.
 #include <cuda_runtime.h>
 
@@ -265,8 +266,9 @@ void enqueue_graph_steps(snn_net *net, int64_t m, cudaStream_t st)
     snn::launch_advance(net->args.ctl, m, st);
 }
 
-// Pipelined engine: m step kernels from the device's t_base, every circuit group in turn, then t_base += m.  Consecutive kernels of a group overlap their launch
-// with the previous one (programmatic edges), inside a captured graph and launched one by
+// Pipelined engine: m step kernels from the device's t_base, every circuit group in turn, then
+// t_base += m.  Consecutive kernels of a group overlap their launch with the previous one
+// (programmatic edges), inside a captured graph and launched one by
 // one alike; a group's first kernel follows the previous group's resync (or the previous
 // run's k_advance, whose t_base it reads before waiting) in plain stream order.
 // One-by-one launches without the edges took 6.2 us per step at pd_full and at pd_tiny,
@@ -947,7 +949,8 @@ int snn_build_network(const snn_spec *spec, void *dev_arena, uint64_t arena_byte
             cuda_ok(cudaMemcpyAsync(A + L.U2, u0.data(), 4 * net->npad, cudaMemcpyHostToDevice, st), "U2");
             cuda_ok(cudaMemsetAsync(A + L.R2, 0, net->npad, st), "R2");
             cuda_ok(cudaMemsetAsync(A + L.queue, 0xFF, 4 * sizeof(snn::QueueEntry) * net->npad, st), "queue");
-            // a graph holds a whole number of phase periods
+            // graphs of any length would do (they take their phase from t_base), but the length that
+            // snn_info reports stays what it always was: a multiple of the phase period
             net->steps_per_graph = std::max(snn::kPhasePeriod,
                                             (spec->steps_per_graph > 0 ? spec->steps_per_graph : 1024) /
                                                 snn::kPhasePeriod * snn::kPhasePeriod);

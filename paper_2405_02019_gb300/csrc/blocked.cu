@@ -21,7 +21,9 @@
 // its own bytes where a copy moves 6.8; BLOCKED4 and 6 of the half-scale circuit 162 -> 107
 // and 192 -> 169 us.  Before, the CTA staged 2,048 senders at a time between barriers, so the
 // record reads drained two or three times per pass.  Short lists are one chain of round trips,
-// list -> bounds -> records -> ring: BLOCKED4 at 2,048 senders 21.5 -> 20.6 us, at 512 10.3 -> 12.2.
+// list -> bounds -> records -> ring, as long as it was (kernel time, BLOCKED4 of the half-scale
+// circuit: 2,048 senders 20.6 -> 20.4 us, 512 10.85 -> 10.8; BLOCKED8 at 512 12.85 -> 11.95).  On
+// few blocks it is longer for BLOCKED4: 52 blocks, 256 to 1,024 senders, 0.3 to 0.6 us of 10 to 20.
 #include <cuda_runtime.h>
 
 #include "internal.hpp"

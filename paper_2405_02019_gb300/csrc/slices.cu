@@ -5,8 +5,8 @@
 // run of it, and all of a list's events with delay d land in one ring row.  A CTA therefore
 // takes a group of delays and a run of senders, sums the events per target in shared
 // memory, and adds each nonzero sum to the ring once.  The row-by-row kernel
-// (k_deliver_list) issues one L2 reduction per event, at random addresses; its rate, about
-// 1.55e11 events per second, is what bounds it, at a fifth of the memory's rate.  Here the
+// (k_deliver_list) issues one L2 reduction per event, at random addresses; their rate, 1.6e11
+// to 1.75e11 events per second, is what bounds it, at a fifth of the memory's rate.  Here the
 // reductions are one per nonzero sum and on consecutive addresses.  The delays of a PLAIN9
 // slice of one delay need not be read at all.
 //   - Shared memory holds kSliceCells sums.  Networks with more neurons are cut into
@@ -20,8 +20,9 @@
 //     them would cost more in clearing and adding the sums than it saves.
 // The records are streamed by independent warps (stream.cuh); a unit is a quad of four
 // records, whose ends outside the slice are masked.
-// Measured (CUDA events, row by row -> slices): 8,192 senders of the half-scale circuit
-// (3.0e7 events) 190 -> 72 us; 20,480 of the full one (7.6e7 events, two parts) 436 -> 229 us.
+// Measured (CUDA events, back to back, one box, row by row -> slices): 8,192 senders (3.0e7
+// events) of the half-scale circuit 191 -> 68 us, of the full one (two parts) 187 -> 110; 20,480
+// (7.6e7 events) 443 -> 141 and 435 -> 227 us.
 #include <cuda_runtime.h>
 
 #include "internal.hpp"
